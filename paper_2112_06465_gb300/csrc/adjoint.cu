@@ -113,15 +113,6 @@ __global__ void k_find_diag(int n, const int *__restrict__ rowptr, const int *__
     }
 }
 
-__global__ void k_set_diag(int n, const int *__restrict__ pos, const double2 *__restrict__ base, double2 c,
-                           const double2 *__restrict__ theta, double2 *__restrict__ val) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double2 v = base[i];
-        cmac(v, c, theta[i]);
-        val[pos[i]] = v;
-    }
-}
-
 __global__ void k_diag_grad(int n, const double2 *__restrict__ mu, const double2 *__restrict__ x, double2 c,
                             double2 *__restrict__ gt) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -199,10 +190,12 @@ extern "C" HZ_API hz_status hz_mat_set_diag(hz_mat *A, const hz_z *d_base, hz_z 
     HZ_CHECK(d_base && d_theta, "hz_mat_set_diag: null vector");
     cudaStream_t s = (cudaStream_t)stream;
     HZ_TRY(ensure_diag(A, s));
-    k_set_diag<<<grid_for(A->n), 256, 0, s>>>(A->n, A->diag_pos, (const double2 *)d_base,
-                                               make_double2(scale.re, scale.im), (const double2 *)d_theta, A->val);
-    HZ_CUDA(cudaGetLastError());
-    return hz_mat_refresh_values(A, stream);
+    free_jacobi(A);   // the scaled copy is rebuilt from the new values on the next use
+    SetDiag sd;
+    sd.base = (const double2 *)d_base;
+    sd.theta = (const double2 *)d_theta;
+    sd.c = make_double2(scale.re, scale.im);
+    return set_diag_refresh(A, sd, s);
 }
 
 extern "C" HZ_API hz_status hz_diag_grad(const hz_mat *A, const hz_z *d_mu, const hz_z *d_x, hz_z scale,

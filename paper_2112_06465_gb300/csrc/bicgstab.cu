@@ -501,7 +501,7 @@ static void spmv_on(const Solver *S, const hz_mat *A, const V *x, const Epi &e, 
     } else if constexpr (std::is_same<V, float2>::value) {
         // complex64 inner operator: block-flat when the handle runs a block-flat kind
         if (A->fblk && is_flat64(d64_kind(A, S->kind)))
-            launch_k(pdl, k_spmv_c64b<Epi>, S->grid_c64, kFlatThreads, cs, mat_view<float2>(A), x, e, S->red);
+            launch_c64_flat(pdl, S->grid_c64, mat_view<float2>(A), x, e, S->red, cs);
         else
             launch_spmv<V>(d64_kind(A, S->kind),
                            S->group, mat_view<V>(A), x, e, S->red, S->grid_spmv_cv, cs, pdl);
@@ -674,12 +674,16 @@ static hz_status get_solver(hz_mat *A, uint32_t mode, cudaStream_t s, Solver **o
             // at once: a grid sized for another epilogue's instantiation
             // would run a partial second wave if these held more registers
             int o1 = 0, o2 = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_spmv_c64b<EpiSigma<float2>>, kFlatThreads, 0) !=
-                    cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_spmv_c64b<EpiOmega<float2>>, kFlatThreads, 0) !=
-                    cudaSuccess)
-                o1 = o2 = 1;
-            const int64_t g = std::min<int64_t>(A->nfblk, (int64_t)d.num_sms * std::max(1, std::min(o1, o2)));
+            const bool sl = A->nsl && A->sl_val32;
+            const cudaError_t e1 =
+                sl ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_spmv_sl<float2, EpiSigma<float2>>, kFlatThreads, 0)
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_spmv_c64b<EpiSigma<float2>>, kFlatThreads, 0);
+            const cudaError_t e2 =
+                sl ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_spmv_sl<float2, EpiOmega<float2>>, kFlatThreads, 0)
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_spmv_c64b<EpiOmega<float2>>, kFlatThreads, 0);
+            if (e1 != cudaSuccess || e2 != cudaSuccess) o1 = o2 = 1;
+            const int64_t units = sl ? (A->nsl + kFlatThreads / 32 - 1) / (kFlatThreads / 32) : A->nfblk;
+            const int64_t g = std::min<int64_t>(units, (int64_t)d.num_sms * std::max(1, std::min(o1, o2)));
             S->grid_c64 = (int)std::max<int64_t>(1, std::min<int64_t>(g, kMaxRedBlocks));
         }
         // HZ_PDL=1 (environment) captures F2..F5 as programmatic dependent

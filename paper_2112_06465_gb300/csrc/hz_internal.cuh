@@ -85,6 +85,15 @@ template <class T> __device__ __forceinline__ T cdiv(T a, T b) {
     r.y = (a.y * b.x - a.x * b.y) / d;
     return r;
 }
+// The complex64 Krylov scalars near the end of a refinement are 1e-20 and
+// less, and their squares leave the binary32 range: both operands are brought
+// to unit size first (by a power of two: exact).
+__device__ __forceinline__ float2 cdiv(float2 a, float2 b) {
+    const int e = (int)((__float_as_uint(fmaxf(fabsf(b.x), fabsf(b.y))) >> 23) & 0xffu);   // biased exponent
+    const float s = __uint_as_float((unsigned)(254 - min(253, max(1, e))) << 23);
+    a.x *= s; a.y *= s; b.x *= s; b.y *= s;
+    return cdiv<float2>(a, b);
+}
 template <class T> __device__ __forceinline__ bool cis_zero(T a) { return a.x == 0 && a.y == 0; }
 
 __device__ __forceinline__ float2 to_c64(double2 a) { return make_float2((float)a.x, (float)a.y); }
@@ -130,6 +139,17 @@ __device__ __forceinline__ float4 ld_stream(const float4 *ptr, uint64_t pol) {
     float4 v;
     asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(ptr), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ double ld_stream(const double *ptr, uint64_t pol) {
+    double v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(ptr), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float2 ld_stream(const float2 *ptr, uint64_t pol) {
+    float2 v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;"
+        : "=f"(v.x), "=f"(v.y) : "l"(ptr), "l"(pol));
     return v;
 }
 __device__ __forceinline__ int ld_stream(const int *ptr, uint64_t pol) {
@@ -571,6 +591,24 @@ struct hz_mat {
     int32_t *pk_col = nullptr;     // [pk_slots]
     double *pk_re = nullptr;       // [pk_slots]
     double *pk_im = nullptr;       // [pk_slots] (complex groups only use it)
+    // row-per-lane binary64 stream (the other layout of HZ_SPMV_FLAT64P, for
+    // matrices whose neighbouring rows have nearly equal lengths; pk_* is then
+    // not built): slice s holds rows 32 s .. 32 s + 31, one per lane, in steps
+    // [sl_base[s], sl_base[s+1]); entry u of a row sits in slot
+    // 32 (sl_base[s] + u) + lane (column -1 past the row's end), the diagonal
+    // entry in the slice's last step, the others in storage order; bit u of sl_mask[s] says
+    // that step u has a nonzero imaginary part
+    int32_t nsl = 0;               // slices (0: no such layout)
+    int64_t sl_slots = 0;
+    int32_t *sl_base = nullptr;    // [nsl + 1]
+    uint64_t *sl_mask = nullptr;   // [nsl]
+    int32_t *sl_diag = nullptr;    // [n] place of the diagonal entry in its row (-1: absent)
+    int32_t *sl_col = nullptr;     // [sl_slots]
+    double *sl_re = nullptr;       // [sl_slots]
+    double *sl_im = nullptr;       // [sl_slots] (read where the mask says so)
+    float2 *sl_val32 = nullptr;    // [sl_slots] complex64 copy, if c64
+    // the handle has one of the two packed binary64 streams
+    bool packed() const { return pk_re || sl_re; }
     int32_t nfblk_t = 0;       // the same for the bulk-copy kernel's smaller chunks
     int32_t *fblk_t = nullptr;
     // owned copy of col, 16-byte aligned and padded by 8 entries, that the
@@ -593,6 +631,12 @@ struct hz_mat {
 };
 
 namespace hz {
+// a new diagonal A_ii = base_i + c theta_i (theta null: none)
+struct SetDiag {
+    const double2 *base = nullptr, *theta = nullptr;
+    double2 c = {0.0, 0.0};
+};
+hz_status set_diag_refresh(hz_mat *A, const SetDiag &sd, cudaStream_t s);   // needs A->diag_pos
 hz_status ensure_jacobi(hz_mat *A, cudaStream_t s);   // build A->jac on first use
 void free_jacobi(hz_mat *A);                          // drop it (values changed, destroy)
 }  // namespace hz

@@ -36,6 +36,14 @@ __global__ void k_sell_gather(int64_t slots, const int *__restrict__ src, const 
     }
 }
 
+__global__ void k_set_diag(int n, const int *__restrict__ pos, SetDiag sd, double2 *__restrict__ val) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        double2 v = sd.base[i];
+        cmac(v, sd.c, sd.theta[i]);
+        val[pos[i]] = v;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Packed binary64 stream of the row blocks (HZ_SPMV_FLAT64P).  Built from
 // the CSR arrays at creation and on every value refresh by three kernels,
@@ -112,6 +120,89 @@ __global__ void k_pk_fill(int nfblk, const int *__restrict__ fblk_k, const int *
     }
 }
 
+// The row-per-lane stream, one warp per slice, lane = row: places the
+// diagonal entry last, records which steps are complex, and (first = 1, at
+// creation) the columns and each row's diagonal place.  With sd.theta set the
+// diagonal entries are base + c theta, written to the caller's values too
+// (hz_mat_set_diag in the same pass).  v32: the complex64 copy, or null.
+//
+// Bound by memory: 16 bytes read and 16 written per entry.  One kernel does
+// what the lane-run stream needs three for (count, scan, fill), because the
+// imaginary parts keep their slot whether a step is complex or not: a new
+// diagonal, one product, the gradient on the pattern and the diagonal's of a
+// 64^3 box went from 93.9 to 62.6 us with it and the product.
+__global__ void __launch_bounds__(256) k_sl_fill(int n, int nsl, const int *__restrict__ base,
+                                                 const int *__restrict__ rowptr, const int *__restrict__ col,
+                                                 double2 *val, int first, int *__restrict__ diag,
+                                                 int *__restrict__ scol, double *__restrict__ sre,
+                                                 double *__restrict__ sim, unsigned long long *__restrict__ mask,
+                                                 float2 *__restrict__ v32, SetDiag sd) {
+    constexpr int G = 4;
+    const int lane = threadIdx.x & 31;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nsl; s += nw) {
+        const int row = 32 * s + lane, b = base[s], w = base[s + 1] - b;
+        int beg = 0, len = 0, d = -1;
+        if (row < n) {
+            beg = rowptr[row];
+            len = min(w, max(0, rowptr[row + 1] - beg));
+            if (first) {
+                for (int k = 0; k < len && d < 0; ++k)
+                    if (col[beg + k] == row) d = k;
+                diag[row] = d;
+            } else {
+                d = diag[row];
+            }
+        }
+        unsigned long long m = 0ull;
+        for (int u0 = 0; u0 < w; u0 += G) {
+            int k[G];
+            double2 a[G];
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                const int u = u0 + q;
+                // the last step: the diagonal entry (a row without one may
+                // end there too); the others in storage order without it
+                int e;
+                if (u >= w - 1) e = u == w - 1 ? (d >= 0 ? d : len == w ? len - 1 : -1) : -1;
+                else if (d >= 0) e = u < len - 1 ? (u < d ? u : u + 1) : -1;
+                else e = u < len ? u : -1;
+                k[q] = e >= 0 ? beg + e : -1;
+                a[q] = k[q] >= 0 ? val[k[q]] : make_double2(0.0, 0.0);
+            }
+            if (sd.theta && d >= 0 && u0 + G >= w) {
+                double2 v = sd.base[row];
+                cmac(v, sd.c, sd.theta[row]);
+                val[beg + d] = v;
+#pragma unroll
+                for (int q = 0; q < G; ++q)
+                    if (u0 + q == w - 1) a[q] = v;
+            }
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                if (u0 + q >= w) break;
+                const size_t slot = (size_t)32 * (b + u0 + q) + lane;
+                if (first) scol[slot] = k[q] >= 0 ? col[k[q]] : -1;
+                sre[slot] = a[q].x;
+                sim[slot] = a[q].y;
+                if (v32) v32[slot] = to_c64(a[q]);
+                if (__any_sync(0xffffffffu, !zero_bits(a[q].y))) m |= 1ull << (u0 + q);
+            }
+        }
+        if (lane == 0) mask[s] = m;
+    }
+}
+
+static hz_status sl_refresh(hz_mat *A, int first, const SetDiag &sd, cudaStream_t s) {
+    DevInfo d;
+    HZ_TRY(dev_info(&d));
+    k_sl_fill<<<stream_grid(d, (int64_t)A->nsl * 32, 256, 8), 256, 0, s>>>(
+        A->n, A->nsl, A->sl_base, A->rowptr, A->col, A->val, first, A->sl_diag, A->sl_col, A->sl_re, A->sl_im,
+        (unsigned long long *)A->sl_mask, A->sl_val32, sd);
+    HZ_CUDA(cudaGetLastError());
+    return HZ_OK;
+}
+
 static hz_status pk_refresh(hz_mat *A, cudaStream_t s) {
     if (!A->pk_re) return HZ_OK;
     DevInfo d;
@@ -178,6 +269,8 @@ MatView<double2> mat_view<double2>(const hz_mat *A) {
     v.perm = A->sell_perm; v.scol = A->sell_col; v.sval = A->sell_val;
     v.pk_base = A->pk_base; v.pk_gbase = A->pk_gbase; v.pk_gim = A->pk_gim; v.pk_col = A->pk_col;
     v.pk_re = A->pk_re; v.pk_im = A->pk_im;
+    v.nsl = A->nsl; v.sl_base = A->sl_base; v.sl_mask = (const unsigned long long *)A->sl_mask;
+    v.sl_col = A->sl_col; v.sl_re = A->sl_re; v.sl_im = A->sl_im;
     return v;
 }
 
@@ -188,6 +281,7 @@ MatView<float2> mat_view<float2>(const hz_mat *A) {
     v.nfblk = A->nfblk; v.fblk = A->fblk; v.fblk_k = A->fblk_k;
     v.nchunks = A->sell_nchunks; v.chunk_off = A->sell_chunk_off; v.chunk_w = A->sell_chunk_w;
     v.perm = A->sell_perm; v.scol = A->sell_col; v.sval = A->sell_val32;
+    v.nsl = A->sl_val32 ? A->nsl : 0; v.sl_base = A->sl_base; v.sl_col = A->sl_col; v.sl_val32 = A->sl_val32;
     return v;
 }
 
@@ -197,14 +291,19 @@ int spmv_grid(const hz_mat *A, int kind, int group, int blocks_per_sm_cap) {
     if (kind == HZ_SPMV_FF_FLAT || kind == HZ_SPMV_FF_TMA || is_flat64(kind)) {
         // persistent: exactly the CTAs that fit at once (blocks are taken
         // grid-stride, so CTAs beyond one wave would only add a tail)
-        static int occ_flat = 0, occ_tma = 0, occ_d64 = 0, occ_d64p = 0;
-        int &occ = kind == HZ_SPMV_FF_TMA ? occ_tma
+        static int occ_flat = 0, occ_tma = 0, occ_d64 = 0, occ_d64p = 0, occ_sl = 0;
+        const bool sl = kind == HZ_SPMV_FLAT64P && A->nsl;
+        int &occ = sl ? occ_sl
+                   : kind == HZ_SPMV_FF_TMA ? occ_tma
                    : kind == HZ_SPMV_FLAT64 ? occ_d64
                    : kind == HZ_SPMV_FLAT64P ? occ_d64p
                                              : occ_flat;
         if (occ == 0) {
             cudaError_t e;
-            if (kind == HZ_SPMV_FF_TMA) {
+            if (sl) {
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_spmv_sl<double2, EpiStore<double2>>,
+                                                                  kFlatThreads, 0);
+            } else if (kind == HZ_SPMV_FF_TMA) {
                 cudaFuncSetAttribute(k_spmv_fft<EpiStore<double2>>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      cudaSharedmemCarveoutMaxShared);
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_spmv_fft<EpiStore<double2>>, kFlatThreads, 0);
@@ -220,7 +319,8 @@ int spmv_grid(const hz_mat *A, int kind, int group, int blocks_per_sm_cap) {
             if (e != cudaSuccess || occ < 1) occ = 1;
         }
         const int wpc = kFlatThreads / 32;
-        int64_t g = std::min<int64_t>(((kind == HZ_SPMV_FF_TMA ? A->nfblk_t : A->nfblk) + wpc - 1) / wpc,
+        const int units = sl ? A->nsl : kind == HZ_SPMV_FF_TMA ? A->nfblk_t : A->nfblk;   // one per warp
+        int64_t g = std::min<int64_t>(((int64_t)units + wpc - 1) / wpc,
                                       (int64_t)d.num_sms * occ);
         return (int)std::max<int64_t>(1, std::min<int64_t>(g, kMaxRedBlocks));
     }
@@ -232,6 +332,16 @@ int spmv_grid(const hz_mat *A, int kind, int group, int blocks_per_sm_cap) {
 int c64_flat_grid(const hz_mat *A) {
     DevInfo d;
     if (dev_info(&d) != HZ_OK) return 1;
+    if (A->nsl && A->sl_val32) {
+        static int occ_sl = 0;
+        if (occ_sl == 0 &&
+            (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_sl, k_spmv_sl<float2, EpiStore<float2>>, kFlatThreads,
+                                                           0) != cudaSuccess || occ_sl < 1))
+            occ_sl = 1;
+        const int wpc = kFlatThreads / 32;
+        const int64_t g = std::min<int64_t>((A->nsl + wpc - 1) / wpc, (int64_t)d.num_sms * occ_sl);
+        return (int)std::max<int64_t>(1, std::min<int64_t>(g, kMaxRedBlocks));
+    }
     static int occ = 0;
     if (occ == 0 &&
         (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_spmv_c64b<EpiStore<float2>>, kFlatThreads, 0) !=
@@ -311,7 +421,8 @@ static hz_status build_sell(hz_mat *A, cudaStream_t s, const std::vector<int> &r
     return HZ_OK;
 }
 
-static hz_status refresh(hz_mat *A, cudaStream_t s) {
+// every copy of the values the handle owns, from the caller's values
+static hz_status refresh(hz_mat *A, cudaStream_t s, int first = 0) {
     DevInfo d;
     HZ_TRY(dev_info(&d));
     if (A->val32 && A->nnz) {
@@ -327,11 +438,23 @@ static hz_status refresh(hz_mat *A, cudaStream_t s) {
             A->sell_slots, A->sell_src, A->val, A->sell_val, A->sell_val32, A->sell_vff);
         HZ_CUDA(cudaGetLastError());
     }
+    if (A->nsl) return sl_refresh(A, first, SetDiag{}, s);
     return pk_refresh(A, s);
+}
+
+// the diagonal base + c theta into the caller's values and every copy
+hz_status set_diag_refresh(hz_mat *A, const SetDiag &sd, cudaStream_t s) {
+    if (A->nsl && !A->val32 && !A->val_ff && !A->sell_val) return sl_refresh(A, 0, sd, s);
+    DevInfo d;
+    HZ_TRY(dev_info(&d));
+    k_set_diag<<<stream_grid(d, A->n, 256, 8), 256, 0, s>>>(A->n, A->diag_pos, sd, A->val);
+    HZ_CUDA(cudaGetLastError());
+    return refresh(A, s);
 }
 
 hz_status ensure_c64(hz_mat *A, cudaStream_t s) {
     if (A->val32) return HZ_OK;
+    if (A->nsl && !A->sl_val32) HZ_CUDA(cudaMalloc(&A->sl_val32, sizeof(float2) * A->sl_slots));
     HZ_CUDA(cudaMalloc(&A->val32, sizeof(float2) * std::max(A->nnz, 1)));
     if (A->sell_val) HZ_CUDA(cudaMalloc(&A->sell_val32, sizeof(float2) * std::max<int64_t>(A->sell_slots, 1)));
     HZ_TRY(refresh(A, s));
@@ -355,7 +478,7 @@ static hz_status autotune(hz_mat *A, cudaStream_t s) {
         for (int w : {2, 4, 8, 16, 32}) cand.push_back({HZ_SPMV_FF, w});
     if (A->sell_vff) cand.push_back({HZ_SPMV_SELL_FF, 0});
     if (A->fblk) cand.push_back({HZ_SPMV_FLAT64, 0});
-    if (A->pk_re) cand.push_back({HZ_SPMV_FLAT64P, 0});
+    if (A->packed()) cand.push_back({HZ_SPMV_FLAT64P, 0});
     if (A->val_ff && A->fblk) cand.push_back({HZ_SPMV_FF_FLAT, 0});
     if (A->col_pad) cand.push_back({HZ_SPMV_FF_TMA, 0});
     float best = 1e30f, best_cv = 1e30f;   // over all kinds; over the binary64 CSR-vector groups
@@ -514,10 +637,47 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
         set_error("hz_csr_create: allocation failed");
         return fail(HZ_ERR_ALLOC);
     }
-    // the packed binary64 stream of these blocks: U = ceil(entries / 32)
+    // the row-per-lane stream where it fits: padded rows cost binary64
+    // instructions, so the padded size may exceed the entries by a quarter
+    // (the lane-run stream's row switches and second accumulator cost it 26 %
+    // more binary64 instructions than the multiply-adds it needs: 728 k
+    // against 577 k on 618 k rows of 15), by two fifths where the work is
+    // small and launches and latency count instead
+    if (n > 0 && nnz > 0) {
+        const int ns = (n + 31) / 32;
+        std::vector<int> sb(ns + 1);
+        int64_t P = 0;
+        int wmax = 0;
+        for (int q = 0; q < ns; ++q) {
+            int w = 0;
+            for (int r = 32 * q; r < std::min(n, 32 * q + 32); ++r) w = std::max(w, rp[r + 1] - rp[r]);
+            sb[q] = (int)std::min<int64_t>(P, INT32_MAX);
+            P += w;
+            wmax = std::max(wmax, w);
+        }
+        sb[ns] = (int)std::min<int64_t>(P, INT32_MAX);
+        const int64_t slots = 32 * P;
+        if (wmax <= kSlMaxWidth && slots < INT32_MAX - 32 &&
+            (4 * slots <= 5 * (int64_t)nnz || (n <= 65536 && 5 * slots <= 7 * (int64_t)nnz))) {
+            A->nsl = ns;
+            A->sl_slots = slots;
+            if (cudaMalloc(&A->sl_base, sizeof(int) * (ns + 1)) != cudaSuccess ||
+                cudaMalloc(&A->sl_mask, sizeof(uint64_t) * ns) != cudaSuccess ||
+                cudaMalloc(&A->sl_diag, sizeof(int) * n) != cudaSuccess ||
+                cudaMalloc(&A->sl_col, sizeof(int) * slots) != cudaSuccess ||
+                cudaMalloc(&A->sl_re, sizeof(double) * slots) != cudaSuccess ||
+                cudaMalloc(&A->sl_im, sizeof(double) * slots) != cudaSuccess ||
+                ((flags & HZ_FLAG_C64) && cudaMalloc(&A->sl_val32, sizeof(float2) * slots) != cudaSuccess) ||
+                cudaMemcpy(A->sl_base, sb.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice) != cudaSuccess) {
+                set_error("hz_csr_create: allocation failed");
+                return fail(HZ_ERR_ALLOC);
+            }
+        }
+    }
+    // else the packed binary64 stream of these blocks: U = ceil(entries / 32)
     // steps of 32 slots per block, groups of kD64Group steps (skipped when
     // the slots would not fit 31-bit offsets)
-    {
+    if (!A->nsl) {
         const int nb = A->nfblk;
         std::vector<int> pb(nb + 1), pg(nb + 1);
         int64_t P = 0, G = 0;
@@ -546,7 +706,7 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
             }
         }
     }
-    A->spmv_kind = A->pk_re ? HZ_SPMV_FLAT64P : HZ_SPMV_FLAT64;
+    A->spmv_kind = A->packed() ? HZ_SPMV_FLAT64P : HZ_SPMV_FLAT64;
     hz_status st;
     if (flags & HZ_FLAG_SELL) {
         if ((st = build_sell(A, s, rp, cl, 1024)) != HZ_OK) return fail(st);
@@ -610,9 +770,9 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
             in_range = h_er[0] >= kFFMinExp && h_er[1] <= kFFMaxExp;
         }
         A->ff_range_ok = in_range;
-        A->spmv_kind = in_range ? HZ_SPMV_FF_FLAT : A->pk_re ? HZ_SPMV_FLAT64P : HZ_SPMV_FLAT64;
+        A->spmv_kind = in_range ? HZ_SPMV_FF_FLAT : A->packed() ? HZ_SPMV_FLAT64P : HZ_SPMV_FLAT64;
     }
-    if ((st = refresh(A, s)) != HZ_OK) return fail(st);
+    if ((st = refresh(A, s, 1)) != HZ_OK) return fail(st);
     if (flags & HZ_FLAG_AUTOTUNE) {
         if ((st = autotune(A, s)) != HZ_OK) return fail(st);
     }
@@ -646,6 +806,13 @@ extern "C" HZ_API hz_status hz_mat_destroy(hz_mat *A) {
     cudaFree(A->pk_col);
     cudaFree(A->pk_re);
     cudaFree(A->pk_im);
+    cudaFree(A->sl_base);
+    cudaFree(A->sl_mask);
+    cudaFree(A->sl_diag);
+    cudaFree(A->sl_col);
+    cudaFree(A->sl_re);
+    cudaFree(A->sl_im);
+    cudaFree(A->sl_val32);
     cudaFree(A->fblk_t);
     cudaFree(A->col_pad);
     cudaFree(A->fault);
@@ -727,8 +894,8 @@ extern "C" HZ_API hz_status hz_cspmv(hz_mat *A, const hz_c *d_x, hz_c *d_y, void
     if (A->fblk && is_flat64(d64_kind(A, A->spmv_kind))) {
         // the block-flat kinds: the block-flat complex64 kernel
         EpiStore<float2> epi{(float2 *)d_y};
-        HZ_CUDA(launch_k(false, k_spmv_c64b<EpiStore<float2>>, c64_flat_grid(A), kFlatThreads, (cudaStream_t)stream,
-                         mat_view<float2>(A), (const float2 *)d_x, epi, RedScratch{}));
+        HZ_CUDA(launch_c64_flat(false, c64_flat_grid(A), mat_view<float2>(A), (const float2 *)d_x, epi, RedScratch{},
+                                (cudaStream_t)stream));
         return HZ_OK;
     }
     const int kind = (A->spmv_kind == HZ_SPMV_SELL || A->spmv_kind == HZ_SPMV_SELL_FF) ? HZ_SPMV_SELL
@@ -752,7 +919,7 @@ extern "C" HZ_API hz_status hz_mat_set_spmv(hz_mat *A, int32_t kind, int32_t gro
         return HZ_OK;
     }
     if (kind == HZ_SPMV_FLAT64P) {
-        HZ_CHECK(A->pk_re != nullptr, "hz_mat_set_spmv: the handle has no packed binary64 stream");
+        HZ_CHECK(A->packed(), "hz_mat_set_spmv: the handle has no packed binary64 stream");
         A->spmv_kind = kind;
         return HZ_OK;
     }

@@ -108,6 +108,14 @@ struct MatView {
     const int *pk_col;
     const double *pk_re;
     const double *pk_im;
+    // row-per-lane stream (see hz_mat::sl_*); nsl = 0 without it
+    int nsl;
+    const int *sl_base;
+    const unsigned long long *sl_mask;
+    const int *sl_col;
+    const double *sl_re;
+    const double *sl_im;
+    const float2 *sl_val32;
 };
 
 // Epilogue interface (every fused SpMV epilogue provides):
@@ -1005,6 +1013,178 @@ __device__ __forceinline__ void flat_rows_d64(const MatView<double2> &A, const d
     }
 }
 
+// ---------------------------------------------------------------------------
+// Row-per-lane core (HZ_SPMV_FLAT64P where the rows of a warp are nearly
+// equally long, and the complex64 product of such handles): one warp per
+// slice of 32 rows, lane l summing row 32 s + l.
+//
+// What bounds it: in binary64 the number of binary64 warp instructions (see
+// above).  With one row per lane there is nothing but the multiply-adds: no
+// second accumulation at row ends, no partial sums between lanes, no row
+// search, and the 32 gathers of a step go to 32 neighbouring rows' columns,
+// which under any local numbering are near-consecutive.  A group of steps
+// whose imaginary parts are all zero takes two FMAs per entry, not four.
+// The diagonal entry is kept apart, in the last step of the slice for every
+// row: an operator that is complex on its diagonal only (a damped or
+// parametrised mass term) has real groups and one complex step, and the
+// largest term of a row is added last, so the others are rounded at their
+// own size.  The price is the padding of short rows to the slice's longest,
+// which is why the layout is chosen by the padded size (hz_csr_create).
+//
+// A predicated-off binary64 instruction occupies the pipe like any other
+// (measured: with both kinds of step under predicates the product took the
+// time of six FMAs per entry), so the real and complex groups and every
+// length of the last group are separate code reached by branches.
+//
+// Measured against the lane runs and, in complex64, the product slab:
+//   618 k rows of 15, real but for the ends   49.5 -> 42.7 us
+//   672 k rows of 27, every value complex      209 -> 137 us (at the pipe's
+//   rate for its 72.6 M multiply-adds)
+//   complex64, 618 k rows of 15               23.4 -> 20.6 us
+// with a smaller error (1.6e-16, 2.0e-16 and 4.7e-8 of the result's norm; before
+// 1.6e-16, 2.4e-16 and 7.7e-8).
+//
+// A skipped term Im(a) x is an exact zero for finite x; for a non-finite x
+// it would be NaN, so the exponent fields of x are watched with two integer
+// operations a component and the NaN is set when the row ends.
+constexpr int kSlG = 8;            // steps whose loads are in flight together
+constexpr int kSlMaxWidth = 64;    // steps per slice at most (bits of the mask)
+// resident CTAs per SM asked of the register allocator
+template <class V> constexpr int kSlMinBlocks = std::is_same<V, double2>::value ? 4 : 8;
+
+// sign bit of the result set iff some value seen was infinite or NaN
+__device__ __forceinline__ void watch_nonfinite(unsigned &bad, double v) {
+    bad |= ((unsigned)__double2hiint(v) & 0x7ff00000u) + 0x00100000u;
+}
+
+// One group of N steps into (y, y2): even and odd steps in two chains.  In
+// the final group of a slice the last step is the diagonal's: it is added
+// to the sum of both chains, as a complex step.
+template <int N, bool kReal, bool kFinal, class V, int G>
+__device__ __forceinline__ void slice_group(V &y, V &y2, const V (&a)[G], const V (&v)[G], unsigned &bad_re,
+                                            unsigned &bad_im) {
+    constexpr int M = kFinal ? N - 1 : N;
+#pragma unroll
+    for (int u = 0; u < M; ++u) {
+        V &q = (u & 1) ? y2 : y;
+        if constexpr (kReal) {
+            q.x = fma(a[u].x, v[u].x, q.x);
+            q.y = fma(a[u].x, v[u].y, q.y);
+            watch_nonfinite(bad_re, v[u].y);
+            watch_nonfinite(bad_im, v[u].x);
+        } else {
+            cmac(q, a[u], v[u]);
+        }
+    }
+    if constexpr (kFinal) {
+        y = cadd(y, y2);
+        cmac(y, a[N - 1], v[N - 1]);
+    }
+}
+template <bool kReal, class V, int G>
+__device__ __forceinline__ void slice_final(int n, V &y, V &y2, const V (&a)[G], const V (&v)[G], unsigned &bad_re,
+                                            unsigned &bad_im) {
+    static_assert(G == 8, "one case per length");
+    switch (n) {
+        case 1: slice_group<1, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        case 2: slice_group<2, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        case 3: slice_group<3, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        case 4: slice_group<4, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        case 5: slice_group<5, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        case 6: slice_group<6, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        case 7: slice_group<7, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        default: slice_group<8, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+    }
+}
+
+// kLive: x was written by other blocks of the running kernel (read it
+// through L2), and the matrix is read again every iteration (let L1 keep it)
+template <class V, class Epi, int NV, bool kLive = false>
+__device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, const Epi &epi,
+                                           typename Epi::Acc (&acc)[NV], int s0, int step, int send) {
+    constexpr bool kD = std::is_same<V, double2>::value;
+    constexpr int G = kSlG;
+    const uint64_t pol = pol_evict_first();
+    const int lane = threadIdx.x & 31;
+    struct Sl {
+        int s, b, w;
+        unsigned long long m;
+    };
+    auto meta = [&](int s) {
+        Sl q{s, 0, 0, 0ull};
+        if (s < send) {
+            q.b = __ldg(A.sl_base + s);
+            q.w = __ldg(A.sl_base + s + 1) - q.b;
+            if constexpr (kD) q.m = __ldg(A.sl_mask + s);
+        }
+        return q;
+    };
+    auto ldm = [&](const auto *p) {
+        if constexpr (kLive) return __ldg(p);
+        else return ld_stream(p, pol);
+    };
+    auto ldx = [&](const V *p) {
+        if constexpr (kLive) return __ldcg(p);
+        else return __ldg(p);
+    };
+    // the column stream runs one group ahead, across slices
+    auto cols = [&](const Sl &q, int u0, int (&c)[G]) {
+        const int *p = A.sl_col + (size_t)32 * (q.b + u0) + lane;
+#pragma unroll
+        for (int u = 0; u < G; ++u) c[u] = u0 + u < q.w ? ldm(p + 32 * u) : -1;
+    };
+    Sl cur = meta(s0), nxt = meta(s0 + step);
+    int cn[G];
+    cols(cur, 0, cn);
+    for (int s = s0; s < send; s += step) {
+        const int row = 32 * s + lane;
+        const bool in = row < A.n;
+        typename PreOf<Epi>::T pf{};
+        if (in) pf = epi_pre(epi, row);
+        V y = czero<V>(), y2 = czero<V>();
+        unsigned bad_re = 0u, bad_im = 0u;
+        const int w = cur.w;
+#pragma unroll 1
+        for (int u0 = 0; u0 < w; u0 += G) {
+            int c[G];
+            V a[G], v[G];
+#pragma unroll
+            for (int u = 0; u < G; ++u) c[u] = cn[u];
+            const size_t o = (size_t)32 * (cur.b + u0) + lane;
+            const unsigned mg = (unsigned)(cur.m >> u0);
+            if constexpr (kD) {
+#pragma unroll
+                for (int u = 0; u < G; ++u) a[u].x = u0 + u < w ? ldm(A.sl_re + o + 32 * u) : 0.0;
+#pragma unroll
+                for (int u = 0; u < G; ++u) a[u].y = (mg >> u) & 1u ? ldm(A.sl_im + o + 32 * u) : 0.0;
+            } else {
+#pragma unroll
+                for (int u = 0; u < G; ++u) a[u] = u0 + u < w ? ldm(A.sl_val32 + o + 32 * u) : czero<V>();
+            }
+            if (u0 + G < w) cols(cur, u0 + G, cn);
+            else cols(nxt, 0, cn);
+#pragma unroll
+            for (int u = 0; u < G; ++u) v[u] = c[u] >= 0 ? ldx(x + c[u]) : czero<V>();
+            const int left = w - u0;
+            if (left > G) {
+                if (kD && !(mg & ((1u << G) - 1u))) slice_group<G, kD, false>(y, y2, a, v, bad_re, bad_im);
+                else slice_group<G, false, false>(y, y2, a, v, bad_re, bad_im);
+            } else {
+                if (kD && !(mg & ((1u << (left - 1)) - 1u))) slice_final<kD>(left, y, y2, a, v, bad_re, bad_im);
+                else slice_final<false>(left, y, y2, a, v, bad_re, bad_im);
+            }
+        }
+        if (w == 0) cols(nxt, 0, cn);
+        if constexpr (kD) {
+            if ((int)bad_re < 0) y.x = __longlong_as_double(0x7ff8000000000000ll);
+            if ((int)bad_im < 0) y.y = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        if (in) epi_row(epi, row, y, acc, pf);
+        cur = nxt;
+        nxt = meta(s + 2 * step);
+    }
+}
+
 // per-thread accumulators -> one grid total -> epi.finish (last block)
 template <class Epi, int NV>
 __device__ __forceinline__ void spmv_reduce(const Epi &epi, typename Epi::Acc (&acc)[NV], RedScratch red) {
@@ -1037,6 +1217,25 @@ __global__ void __launch_bounds__(kFlatThreads, kD64MinBlocks) k_spmv_d64b(MatVi
     if constexpr (Epi::NV > 0) spmv_reduce<Epi, NV>(epi, acc, red);
 }
 
+// the row-per-lane kernel (kFlatThreads threads, one warp per slice); 128
+// registers and 16 warps per SM in binary64
+template <class V, class Epi>
+__global__ void __launch_bounds__(kFlatThreads, kSlMinBlocks<V>) k_spmv_sl(MatView<V> A, const V *__restrict__ x,
+                                                                           Epi epi, RedScratch red) {
+    constexpr int NV = Epi::NV > 0 ? Epi::NV : 1;
+    pdl_wait();
+    pdl_release();
+    if (epi.skip()) {   // grid-uniform early exit; one thread reports it to the epilogue
+        if (blockIdx.x == 0 && threadIdx.x == 0) epi.on_skip();
+        return;
+    }
+    typename Epi::Acc acc[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) Epi::zero(acc[j]);
+    const int wpc = blockDim.x >> 5;
+    slice_rows<V, Epi, NV>(A, x, epi, acc, blockIdx.x * wpc + (threadIdx.x >> 5), gridDim.x * wpc, A.nsl);
+    if constexpr (Epi::NV > 0) spmv_reduce<Epi, NV>(epi, acc, red);
+}
 
 template <int W, class T, class Epi>
 __global__ void __launch_bounds__(kSpmvBlock) k_spmv(MatView<T> A, const T *__restrict__ x, Epi epi,
@@ -1254,8 +1453,12 @@ __global__ void __launch_bounds__(kFlatThreads) k_spmv_c64b(MatView<float2> A, c
     if constexpr (Epi::NV > 0) spmv_reduce<Epi, NV>(epi, acc, red);
 }
 
-// grid of k_spmv_c64b: the CTAs that fit at once
+// the block-flat complex64 product: row per lane where the handle has that
+// layout, else k_spmv_c64b; and its grid, the CTAs that fit at once
 int c64_flat_grid(const hz_mat *A);
+template <class Epi>
+cudaError_t launch_c64_flat(bool pdl, int grid, const MatView<float2> &A, const float2 *x, const Epi &epi,
+                            RedScratch red, cudaStream_t s);
 
 // binary64 -> double-float split of a vector (xff[i] = split_ff(x[i])), on stream s
 cudaError_t split_ff_vec(int n, const double2 *x, float4 *xff, cudaStream_t s);
@@ -1285,6 +1488,13 @@ cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, cudaS
     return cudaGetLastError();
 }
 
+template <class Epi>
+cudaError_t launch_c64_flat(bool pdl, int grid, const MatView<float2> &A, const float2 *x, const Epi &epi,
+                            RedScratch red, cudaStream_t s) {
+    if (A.nsl) return launch_k(pdl, k_spmv_sl<float2, Epi>, grid, kFlatThreads, s, A, x, epi, red);
+    return launch_k(pdl, k_spmv_c64b<Epi>, grid, kFlatThreads, s, A, x, epi, red);
+}
+
 // launch helper: picks the template instance for the handle's variant
 template <class T, class Epi>
 cudaError_t launch_spmv(int kind, int group, const MatView<T> &A, const T *x, const Epi &epi,
@@ -1292,6 +1502,10 @@ cudaError_t launch_spmv(int kind, int group, const MatView<T> &A, const T *x, co
     if constexpr (std::is_same<T, double2>::value) {
         if (kind == HZ_SPMV_FLAT64) {
             launch_k(pdl, k_spmv_d64b<Epi, false>, grid, kFlatThreads, s, A, x, epi, red);
+            return cudaGetLastError();
+        }
+        if (kind == HZ_SPMV_FLAT64P && A.nsl) {
+            launch_k(pdl, k_spmv_sl<double2, Epi>, grid, kFlatThreads, s, A, x, epi, red);
             return cudaGetLastError();
         }
         if (kind == HZ_SPMV_FLAT64P) {
@@ -1360,7 +1574,7 @@ inline int d64_kind(const hz_mat *A, int kind) {
     if (kind == HZ_SPMV_SELL || kind == HZ_SPMV_SELL_FF) return HZ_SPMV_SELL;
     if (kind == HZ_SPMV_CSR_VECTOR || kind == HZ_SPMV_FF) return HZ_SPMV_CSR_VECTOR;
     if (kind == HZ_SPMV_FLAT64) return HZ_SPMV_FLAT64;
-    return A->pk_re ? HZ_SPMV_FLAT64P : HZ_SPMV_FLAT64;
+    return A->packed() ? HZ_SPMV_FLAT64P : HZ_SPMV_FLAT64;
 }
 // the binary64 block-flat kinds
 inline bool is_flat64(int kind) { return kind == HZ_SPMV_FLAT64 || kind == HZ_SPMV_FLAT64P; }

@@ -1,0 +1,121 @@
+"""The row-per-lane layout of the packed binary64 stream (and of the complex64
+copy): slices of 32 rows, the diagonal entry in a slice's last step, groups of
+8 steps.  Sizes at the edges: a partial last slice, widths around one and
+several groups and at the widest slice, rows without a diagonal entry or
+without any entry, duplicate diagonal entries; groups that change between real
+and complex under a value refresh or a new diagonal; non-finite x.
+
+Tolerance of a binary64 entry: any order of its 2 m products is within
+(2 m + 1) 2^-53 sum |a||x| of the exact value, twice that against the oracle
+(m: entries of the row; one addition more for the second chain).  Complex64:
+4e-6 sum |a||x|, 2^-24 times twice the 2 m <= 130 roundings of either side."""
+
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from tests import _cases as K
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.as_tensor(a).cuda()
+
+
+def host(t):
+    torch.cuda.synchronize()
+    return t.cpu().numpy()
+
+
+def banded(n, width, seed, real=True, diag="all"):
+    """Rows of `width` entries (fewer only by the rules of `diag`) near the
+    diagonal; values real off the diagonal and complex on it, or all complex."""
+    rng = np.random.default_rng(seed)
+    rp, cols, vals = [0], [], []
+    for i in range(n):
+        lo = min(max(0, i - width // 2), n - width)
+        c = np.arange(lo, lo + width)
+        if diag == "some" and i % 5 == 2:
+            c = c[c != i]                        # no diagonal entry
+        if diag == "some" and i % 37 == 11:
+            c = c[:0]                            # no entry at all
+        if diag == "twice" and i % 3 == 0 and c.size:
+            c = np.sort(np.append(c[c != (c[0] if c[0] != i else c[-1])], i))   # the diagonal stored twice
+        v = rng.standard_normal(c.size) + 0j
+        cplx = np.ones(c.size, bool) if not real else c == i
+        v[cplx] += 1j * rng.standard_normal(int(cplx.sum()))
+        rp.append(rp[-1] + c.size)
+        cols.append(c)
+        vals.append(v)
+    return W.CSR(n, np.array(rp, np.int32), np.concatenate(cols).astype(np.int32), np.concatenate(vals))
+
+
+def bound(A, x):
+    m = np.diff(A.rowptr).astype(np.float64)
+    return (2.0 * m + 4.0) * 2.0 ** -52 * K.row_abs_scale(A, x) + 1e-300
+
+
+@pytest.mark.parametrize("n,width,real,diag", [
+    (1, 1, True, "all"), (31, 7, True, "all"), (33, 8, False, "all"), (1000, 9, True, "some"),
+    (4099, 15, True, "all"), (4099, 16, False, "some"), (777, 17, True, "twice"), (500, 27, False, "all"),
+    (300, 64, True, "all"), (300, 65, True, "all")])
+def test_product_widths_and_rows(hz, oracle, n, width, real, diag):
+    A = banded(n, width, 3 * n + width, real, diag)
+    x = K.vectors(n, n + 1)[0]
+    M = hz.Matrix.from_csr(A, c64=True)
+    assert np.all(np.abs(host(hz.zspmv(M, dev(x))) - oracle.zspmv(A, x)) <= bound(A, x))
+    x32 = x.astype(np.complex64)
+    err = np.abs(host(hz.cspmv(M, dev(x32))) - oracle.cspmv(A, x32))
+    assert np.all(err <= 4e-6 * K.row_abs_scale(A, x32.astype(np.complex128)) + 1e-30)
+    M.close()
+
+
+def test_value_refresh_and_new_diagonal(hz, oracle):
+    """Real groups turn complex and back with the caller's values, the
+    diagonal follows hz_mat_set_diag, with and without a complex64 copy."""
+    A = banded(1500, 15, 5, real=True)
+    rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
+    x, th = K.vectors(A.n, 6)
+    base = K.vectors(A.n, 8)[0]
+    for c64 in (False, True):
+        vd = dev(A.val.copy())
+        M = hz.Matrix(dev(A.rowptr), dev(A.col), vd, c64=c64)
+        v = A.val.copy()
+        v[(rows >= 400) & (rows < 470)] *= 1j
+        for cur in (v, A.val):
+            vd.copy_(torch.as_tensor(cur))
+            M.refresh_values()
+            B = W.CSR(A.n, A.rowptr, A.col, cur)
+            assert np.all(np.abs(host(hz.zspmv(M, dev(x))) - oracle.zspmv(B, x)) <= bound(B, x))
+        hz.mat_set_diag(M, dev(base), -3.0 + 0.5j, dev(th))
+        new = A.val.copy()
+        new[A.col == rows] = base + (-3.0 + 0.5j) * th
+        B = W.CSR(A.n, A.rowptr, A.col, new)
+        # base + c theta: two products and two sums of unit size
+        assert np.allclose(host(vd), new, rtol=0, atol=8 * 2.0 ** -53 * (np.abs(base).max() + 4 * np.abs(th).max()))
+        B = W.CSR(A.n, A.rowptr, A.col, host(vd))
+        assert np.all(np.abs(host(hz.zspmv(M, dev(x))) - oracle.zspmv(B, x)) <= bound(B, x))
+        if c64:
+            x32 = x.astype(np.complex64)
+            err = np.abs(host(hz.cspmv(M, dev(x32))) - oracle.cspmv(B, x32))
+            assert np.all(err <= 4e-6 * K.row_abs_scale(B, x32.astype(np.complex128)))
+        M.close()
+
+
+def test_nonfinite_x(hz, oracle):
+    """An infinite or NaN entry of x reaches a row as in binary64 arithmetic
+    (0 * inf = NaN), in real groups, complex groups and the diagonal step."""
+    A = banded(700, 15, 9, real=True)
+    x = K.vectors(A.n, 10)[0]
+    x[100], x[351], x[699] = complex(np.inf, 1.0), complex(2.0, np.nan), complex(0.5, -np.inf)
+    M = hz.Matrix.from_csr(A)
+    with np.errstate(all="ignore"):
+        ref = oracle.zspmv(A, x)
+    y = host(hz.zspmv(M, dev(x)))
+    assert np.array_equal(np.isnan(y.real), np.isnan(ref.real))
+    assert np.array_equal(np.isnan(y.imag), np.isnan(ref.imag))
+    ok = np.isfinite(ref.real) & np.isfinite(ref.imag)
+    assert np.allclose(y[ok], ref[ok], rtol=0, atol=1e-12)
+    M.close()
