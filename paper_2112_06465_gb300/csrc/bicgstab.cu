@@ -27,7 +27,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "krylov.cuh"
+#include "persist.cuh"
 
 namespace hz {
 
@@ -446,6 +446,10 @@ void free_solvers(hz_mat *A) {
     A->solver_bl = nullptr;
     tq_solver_free(A->solver_tq);
     A->solver_tq = nullptr;
+    for (void *&q : A->solver_ps) {
+        ps_solver_free(q);
+        q = nullptr;
+    }
 }
 
 #define HZ_ALLOC(ptr, bytes) HZ_CUDA(cudaMalloc((void **)&(ptr), std::max<size_t>((bytes), 16)))
@@ -747,16 +751,22 @@ extern "C" HZ_API hz_status hz_zsolve_opts(hz_mat *A, const hz_z *d_b, hz_z *d_x
     c.pre_d = op != A ? A->jac_d : nullptr;
     c.pre_dinv = op != A ? A->jac_dinv : nullptr;
     c.op_scale = 1.0;
-    if (o->method == HZ_METHOD_BICGSTABL || o->method == HZ_METHOD_TFQMR) {
+    // systems whose vectors fit on chip: one persistent kernel
+    const PsKind pk = o->method == HZ_METHOD_TFQMR ? PS_TFQMR : o->mode == HZ_MODE_MIXED ? PS_MIXED : PS_BICG;
+    const bool ps = o->method != HZ_METHOD_BICGSTABL && ps_fits(op, pk);
+    if (ps || o->method == HZ_METHOD_BICGSTABL || o->method == HZ_METHOD_TFQMR) {
         Info inf{};
         int restarts = 0;
-        if (o->method == HZ_METHOD_BICGSTABL) HZ_TRY(bl_solve(op, o->ell, c, &inf, &restarts, s));
+        if (ps) {
+            if (pk == PS_MIXED) HZ_TRY(ensure_c64(op, s));
+            HZ_TRY(ps_solve(op, pk, c, &inf, &restarts, s));
+        } else if (o->method == HZ_METHOD_BICGSTABL) HZ_TRY(bl_solve(op, o->ell, c, &inf, &restarts, s));
         else HZ_TRY(tq_solve(op, c, &inf, &restarts, s));
         if (inf.status == HZ_OK && inf.relres_true > o->tol) inf.status = HZ_NOT_CONVERGED;
         h_info->iters = inf.iters;
         h_info->status = inf.status;
         h_info->restarts = restarts;
-        h_info->outer = 0;
+        h_info->outer = inf.outer;
         h_info->relres_rec = inf.relres_rec;
         h_info->relres_true = inf.relres_true;
         return (hz_status)inf.status;

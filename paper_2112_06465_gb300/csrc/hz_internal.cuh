@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string>
+#include <vector>
 
 #include "../../include/hz.h"
 
@@ -155,6 +156,19 @@ __device__ __forceinline__ float2 ld_stream(const float2 *ptr, uint64_t pol) {
 __device__ __forceinline__ int ld_stream(const int *ptr, uint64_t pol) {
     int v;
     asm("ld.global.nc.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(ptr), "l"(pol));
+    return v;
+}
+
+// loads of data that other blocks of the running kernel wrote (through L2;
+// volatile: neither merged nor moved across a barrier)
+__device__ __forceinline__ double2 ld_live(const double2 *p) {
+    double2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_live(const float2 *p) {
+    float2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
     return v;
 }
 
@@ -601,6 +615,7 @@ struct hz_mat {
     int32_t nsl = 0;               // slices (0: no such layout)
     int64_t sl_slots = 0;
     int32_t *sl_base = nullptr;    // [nsl + 1]
+    std::vector<int32_t> sl_base_h;   // the same on the host
     uint64_t *sl_mask = nullptr;   // [nsl]
     int32_t *sl_diag = nullptr;    // [n] place of the diagonal entry in its row (-1: absent)
     int32_t *sl_col = nullptr;     // [sl_slots]
@@ -622,6 +637,7 @@ struct hz_mat {
     void *solver[2] = {nullptr, nullptr};
     void *solver_bl = nullptr;
     void *solver_tq = nullptr;
+    void *solver_ps[3] = {nullptr, nullptr, nullptr};   // persistent solvers (PsKind)
     // Jacobi right preconditioning: the column-scaled operator A D^-1 as a
     // handle of its own (borrowing rowptr/col), its values, and D, D^-1
     hz_mat *jac = nullptr;

@@ -80,6 +80,34 @@ struct BiState {
 
 template <class V> using StateOf = BiState<typename Ar<V>::St>;
 
+// TFQMR's scalars beside the state (tfqmr.cu)
+struct TqExtra {
+    double2 eta;       // eta of the last half step
+    double2 coef1, eta1, coef2, eta2;   // d/x coefficients of the two half steps of this iteration
+    double tau, theta;
+    double xs;         // 1 / G: x moves by eta * xs * d (vectors held scaled by G <= 1)
+    double2 eta1x, eta2x;   // eta1 * xs, eta2 * xs
+    int m;             // half steps since the (re)start
+    int stop;          // the stopping test fired: finish the pending x update, then stop
+    int pend;          // rescale by 2^-64 at the start of the next iteration
+};
+
+constexpr double kTqBig = 1.329227995784916e36;     // 2^120: rescale threshold for squared norms
+constexpr double kTqShrink = 5.421010862427522e-20;  // 2^-64
+
+// one half step's scalars from ||w||^2 (single thread)
+__device__ __forceinline__ void tq_half_step(double2 alpha, TqExtra *q, double ww, double2 &coef, double2 &eta_h) {
+    q->m += 1;
+    const double th_prev = q->theta;
+    const double theta = q->tau == 0.0 ? 0.0 : sqrt(ww) / q->tau;
+    const double c = 1.0 / sqrt(1.0 + theta * theta);
+    q->tau = q->tau * theta * c;
+    coef = cdiv(make_double2(th_prev * th_prev * q->eta.x, th_prev * th_prev * q->eta.y), alpha);
+    eta_h = make_double2(c * c * alpha.x, c * c * alpha.y);
+    q->eta = eta_h;
+    q->theta = theta;
+}
+
 struct OuterState {   // mixed-precision refinement state
     double nb, rel;
     double rel_best;  // smallest outer residual ratio so far (its iterate is in the best-x vector)

@@ -1,0 +1,17 @@
+// persist.cuh -- the persistent single-kernel solvers (persist.cu)
+#pragma once
+
+#include "krylov.cuh"
+
+namespace hz {
+
+enum PsKind { PS_BICG = 0, PS_MIXED = 1, PS_TFQMR = 2 };
+
+// whether a solve on this handle runs as one persistent kernel: a binary64
+// handle in the row-per-lane layout, the Krylov vectors of its rows within
+// the shared memory of the GPU's SMs
+bool ps_fits(const hz_mat *A, PsKind k);
+hz_status ps_solve(hz_mat *A, PsKind kind, const Ctl &c, Info *out, int *restarts, cudaStream_t s);
+void ps_solver_free(void *p);
+
+}  // namespace hz

@@ -661,6 +661,7 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
             (4 * slots <= 5 * (int64_t)nnz || (n <= 65536 && 5 * slots <= 7 * (int64_t)nnz))) {
             A->nsl = ns;
             A->sl_slots = slots;
+            A->sl_base_h.assign(sb.begin(), sb.end());
             if (cudaMalloc(&A->sl_base, sizeof(int) * (ns + 1)) != cudaSuccess ||
                 cudaMalloc(&A->sl_mask, sizeof(uint64_t) * ns) != cudaSuccess ||
                 cudaMalloc(&A->sl_diag, sizeof(int) * n) != cudaSuccess ||

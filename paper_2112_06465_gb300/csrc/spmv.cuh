@@ -1097,11 +1097,18 @@ __device__ __forceinline__ void slice_final(int n, V &y, V &y2, const V (&a)[G],
     }
 }
 
-// kLive: x was written by other blocks of the running kernel (read it
-// through L2), and the matrix is read again every iteration (let L1 keep it)
-template <class V, class Epi, int NV, bool kLive = false>
+struct NoWait {
+    __device__ bool operator()() const { return true; }
+};
+// kLive: 1: x was written by other blocks of the running kernel (read it
+// through L2), and the matrix is read again every iteration (let L1 keep it);
+// 2: and the slices s0 .. send of the stream are in shared memory.
+// wait() runs once on every thread after the first columns are requested and
+// before x is read; the rows are left out if it returns false.
+template <class V, class Epi, int NV, int kLive = 0, class Wait = NoWait>
 __device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, const Epi &epi,
-                                           typename Epi::Acc (&acc)[NV], int s0, int step, int send) {
+                                           typename Epi::Acc (&acc)[NV], int s0, int step, int send,
+                                           Wait wait = Wait{}) {
     constexpr bool kD = std::is_same<V, double2>::value;
     constexpr int G = kSlG;
     const uint64_t pol = pol_evict_first();
@@ -1113,18 +1120,25 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, cons
     auto meta = [&](int s) {
         Sl q{s, 0, 0, 0ull};
         if (s < send) {
-            q.b = __ldg(A.sl_base + s);
-            q.w = __ldg(A.sl_base + s + 1) - q.b;
-            if constexpr (kD) q.m = __ldg(A.sl_mask + s);
+            if constexpr (kLive == 2) {
+                q.b = A.sl_base[s];
+                q.w = A.sl_base[s + 1] - q.b;
+                if constexpr (kD) q.m = A.sl_mask[s];
+            } else {
+                q.b = __ldg(A.sl_base + s);
+                q.w = __ldg(A.sl_base + s + 1) - q.b;
+                if constexpr (kD) q.m = __ldg(A.sl_mask + s);
+            }
         }
         return q;
     };
     auto ldm = [&](const auto *p) {
-        if constexpr (kLive) return __ldg(p);
+        if constexpr (kLive == 2) return *p;
+        else if constexpr (kLive == 1) return __ldg(p);
         else return ld_stream(p, pol);
     };
     auto ldx = [&](const V *p) {
-        if constexpr (kLive) return __ldcg(p);
+        if constexpr (kLive != 0) return ld_live(p);
         else return __ldg(p);
     };
     // the column stream runs one group ahead, across slices
@@ -1136,6 +1150,7 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, cons
     Sl cur = meta(s0), nxt = meta(s0 + step);
     int cn[G];
     cols(cur, 0, cn);
+    if (!wait()) return;
     for (int s = s0; s < send; s += step) {
         const int row = 32 * s + lane;
         const bool in = row < A.n;

@@ -32,34 +32,6 @@
 
 namespace hz {
 
-struct TqExtra {
-    double2 eta;       // eta of the last half step
-    double2 coef1, eta1, coef2, eta2;   // d/x coefficients of the two half steps of this iteration
-    double tau, theta;
-    double xs;         // 1 / G: x moves by eta * xs * d (vectors held scaled by G <= 1)
-    double2 eta1x, eta2x;   // eta1 * xs, eta2 * xs
-    int m;             // half steps since the (re)start
-    int stop;          // the stopping test fired: finish the pending x update, then stop
-    int pend;          // rescale by 2^-64 at the start of the next iteration
-};
-
-constexpr double kTqBig = 1.329227995784916e36;     // 2^120: rescale threshold for squared norms
-constexpr double kTqShrink = 5.421010862427522e-20;  // 2^-64
-
-// one half step's scalars from ||w||^2 (single thread)
-__device__ __forceinline__ void tq_half_step(StateOf<double2> *st, TqExtra *q, double ww, double2 &coef,
-                                             double2 &eta_h) {
-    q->m += 1;
-    const double th_prev = q->theta;
-    const double theta = q->tau == 0.0 ? 0.0 : sqrt(ww) / q->tau;
-    const double c = 1.0 / sqrt(1.0 + theta * theta);
-    q->tau = q->tau * theta * c;
-    coef = cdiv(make_double2(th_prev * th_prev * q->eta.x, th_prev * th_prev * q->eta.y), st->alpha);
-    eta_h = make_double2(c * c * st->alpha.x, c * c * st->alpha.y);
-    q->eta = eta_h;
-    q->theta = theta;
-}
-
 // start epilogue: w = u1 = r^ = b - A x, d = v = 0, ||r||^2, ||b||^2
 template <class V>
 struct EpiTqInit : EpiBase<V> {
@@ -191,7 +163,7 @@ __global__ void __launch_bounds__(kVecBlock) k_tq_half1(int n, StateOf<V> *st, T
             st->rho = make_double2(st->rho.x * kTqShrink, st->rho.y * kTqShrink);
             q->xs /= kTqShrink;
         }
-        tq_half_step(st, q, (double)tot[0], q->coef1, q->eta1);
+        tq_half_step(st->alpha, q, (double)tot[0], q->coef1, q->eta1);
         q->eta1x = make_double2(q->eta1.x * q->xs, q->eta1.y * q->xs);
     }
 }
@@ -221,7 +193,7 @@ struct EpiTqW : EpiBase<V> {
         A::dotc(acc[1], acc[2], rh[i], wi);
     }
     template <int N> __device__ void finish(R (&tot)[N]) const {
-        tq_half_step(st, q, (double)tot[0], q->coef2, q->eta2);
+        tq_half_step(st->alpha, q, (double)tot[0], q->coef2, q->eta2);
         q->eta2x = make_double2(q->eta2.x * q->xs, q->eta2.y * q->xs);
         const int it = st->iter + 1;
         st->iter = it;

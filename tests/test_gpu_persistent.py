@@ -1,0 +1,106 @@
+"""Solves as one persistent kernel (systems in the row-per-lane layout whose
+vectors fit on chip) against the same solve on the graph of kernels, which a
+handle switched to the unpacked kind takes: every method, sizes from one row to
+the largest that fits and the first that does not, partial slices, CTAs that
+own no, one or several slices, a matrix staged in shared memory or not.
+
+The operator is diagonally dominant: A = d I + B with |d| >= 4 and row and
+column sums of |B| at most 1, so ||A|| <= 5.2 and ||A^-1|| <= 1/3.  Two
+solutions of relative residual tol differ by at most 2 tol ||A^-1|| ||b||, and
+||b|| <= 5.2 ||x||: 3.5 tol ||x||."""
+
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-11
+
+
+def operator(n, seed, bands=(1, 7, 40)):
+    """Diagonal 4 + i and off-diagonals at the distances `bands`, of sizes
+    whose sum over a row or a column is at most 1, some of them complex."""
+    rng = np.random.default_rng(seed)
+    off = [o for k in bands if k < n for o in (-k, k)]
+    i = np.arange(n)
+    cols, vals = [i], [np.full(n, 4.0 + 1.0j)]
+    for o in off:
+        c = i + o
+        v = rng.uniform(-1, 1, n) / max(1, len(off)) + 0j
+        if o == off[-1]:
+            v[n // 2:] *= 1j
+        cols.append(c)
+        vals.append(v)
+    c, v = np.stack(cols, 1), np.stack(vals, 1)
+    ok = (c >= 0) & (c < n)
+    order = np.argsort(np.where(ok, c, n + 1), axis=1, kind="stable")
+    c, v, ok = (np.take_along_axis(q, order, 1) for q in (c, v, ok))
+    rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+    return W.CSR(n, rp, c[ok].astype(np.int32), v[ok])
+
+
+def vec(n, seed):
+    rng = np.random.default_rng(seed)
+    return torch.as_tensor(rng.standard_normal(n) + 1j * rng.standard_normal(n)).cuda()
+
+
+METHODS = [dict(method="bicgstab"), dict(method="tfqmr"), dict(mode="mixed"),
+           dict(method="bicgstab", precond="jacobi"), dict(method="tfqmr", precond="jacobi")]
+# 152 x 32 = 4864 rows give every SM one slice; 60 x 4864 is the most that
+# BiCGStab in binary64 holds on chip, 47 x 4864 TFQMR
+SIZES = [1, 2, 31, 33, 1000, 4864, 4865, 20011, 100003, 47 * 4864, 60 * 4864, 60 * 4864 + 1]
+
+
+@pytest.mark.parametrize("n", SIZES)
+def test_persistent_against_graph(hz, n):
+    A = operator(n, n)
+    b, x0 = vec(n, n + 1), vec(n, n + 2)
+    for opt in METHODS if n <= 20011 else METHODS[:3]:
+        sols = []
+        for kind in ("flat64p", "flat64"):
+            M = hz.Matrix.from_csr(A, c64=True)
+            M.set_spmv(kind)
+            hist = torch.zeros(201, dtype=torch.float64, device="cuda")
+            x, info = hz.zsolve(M, b, x=x0.clone(), tol=TOL, maxit=200, hist=hist, **opt)
+            assert info.status == 0 and info.relres_true <= TOL, (kind, opt, info)
+            r = b - hz.zspmv(M, x)
+            # b - A x again: rounding of both evaluations, (2 m + 4) 2^-52 of |A||x| + |b|
+            assert abs(float(torch.linalg.vector_norm(r) / torch.linalg.vector_norm(b)) - info.relres_true) <= 2e-14
+            sols.append((x, info, hist))
+            M.close()
+        (xa, ia, ha), (xb, ib, hb) = sols
+        d = float(torch.linalg.vector_norm(xa - xb) / torch.linalg.vector_norm(xb))
+        assert d <= 3.5 * TOL, (opt, d)
+        assert abs(ia.iters - ib.iters) <= 2 + ib.iters // 4
+        # the start's residual: sums in another order, n terms
+        assert abs(float(ha[0] - hb[0])) <= 1e-12 * float(hb[0])
+
+
+@pytest.mark.parametrize("opt", METHODS[:3])
+def test_outcomes(hz, opt):
+    n = 5000
+    M = hz.Matrix.from_csr(operator(n, 3), c64=True)
+    b, zero = vec(n, 4), torch.zeros(n, dtype=torch.complex128, device="cuda")
+    x, info = hz.zsolve(M, zero, x=vec(n, 5), tol=TOL, maxit=50, **opt)
+    assert info.status == 0 and info.iters == 0 and not bool(x.any())
+    x, info = hz.zsolve(M, b, tol=TOL, maxit=0, **opt)
+    assert info.status == 4 and info.iters == 0 and not bool(x.any())
+    x, info = hz.zsolve(M, b, tol=1e-30, maxit=3, **opt)
+    assert info.status == 4 and info.iters == 3
+    bad = b.clone()
+    bad[777] = complex(float("nan"), 0.0)
+    x, info = hz.zsolve(M, bad, tol=TOL, maxit=50, **opt)
+    assert info.status == 6
+    x, info = hz.zsolve(M, b, tol=TOL, maxit=50, **opt)      # and the handle still solves
+    assert info.status == 0
+    y, again = hz.zsolve(M, b, tol=TOL, maxit=50, **opt)     # deterministic
+    assert torch.equal(x, y) and again.iters == info.iters
+    # a right-hand side whose squares are near the ends of the binary64 range
+    for s in (2.0 ** -480, 2.0 ** 440):
+        if opt.get("mode") != "mixed":
+            z, info = hz.zsolve(M, b * s, tol=TOL, maxit=50, **opt)
+            assert info.status == 0
+            assert float(torch.linalg.vector_norm(z / s - x) / torch.linalg.vector_norm(x)) <= 3.5 * TOL
+    M.close()
