@@ -446,6 +446,8 @@ void free_solvers(hz_mat *A) {
     A->solver_bl = nullptr;
     tq_solver_free(A->solver_tq);
     A->solver_tq = nullptr;
+    ps_batch_free(A->ps_batch);
+    A->ps_batch = nullptr;
     for (void *&q : A->solver_ps) {
         ps_solver_free(q);
         q = nullptr;

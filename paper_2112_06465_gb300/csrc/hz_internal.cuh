@@ -638,6 +638,7 @@ struct hz_mat {
     void *solver_bl = nullptr;
     void *solver_tq = nullptr;
     void *solver_ps[3] = {nullptr, nullptr, nullptr};   // persistent solvers (PsKind)
+    void *ps_batch = nullptr;                            // workspace of sweeps that begin with this handle
     // Jacobi right preconditioning: the column-scaled operator A D^-1 as a
     // handle of its own (borrowing rowptr/col), its values, and D, D^-1
     hz_mat *jac = nullptr;

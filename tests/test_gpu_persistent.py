@@ -104,3 +104,24 @@ def test_outcomes(hz, opt):
             assert info.status == 0
             assert float(torch.linalg.vector_norm(z / s - x) / torch.linalg.vector_norm(x)) <= 3.5 * TOL
     M.close()
+
+
+@pytest.mark.parametrize("sizes", [(4000,), (33, 20011, 1, 700), (300,) * 152, (300,) * 153, (290000, 40000)])
+def test_sweep_against_single_solves(hz, sizes):
+    """A sweep shares the SMs out among its systems (153 systems, and two that
+    do not fit together, take the grid-wide phases); a start vector is used,
+    and a zero right-hand side leaves it."""
+    mats = [hz.Matrix.from_csr(operator(n, 7 + k)) for k, n in enumerate(sizes)]
+    bs = [vec(n, 50 + k) for k, n in enumerate(sizes)]
+    xs = [vec(n, 300 + k) for k, n in enumerate(sizes)]
+    if len(sizes) == 4:
+        bs[3].zero_()
+        keep = xs[3].clone()
+    xs, infos = hz.zsolve_batched(mats, bs, xs=xs, tol=TOL, maxit=200)
+    for k, (M, b, x, info) in enumerate(zip(mats, bs, xs, infos)):
+        assert info.status == 0, (k, info)
+        if len(sizes) == 4 and k == 3:
+            assert info.iters == 0 and torch.equal(x, keep)
+        elif k < 4:
+            y, _ = hz.zsolve(M, b, tol=TOL, maxit=200)
+            assert float(torch.linalg.vector_norm(x - y) / torch.linalg.vector_norm(y)) <= 3.5 * TOL
