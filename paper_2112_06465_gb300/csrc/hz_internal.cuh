@@ -172,6 +172,29 @@ __device__ __forceinline__ float2 ld_live(const float2 *p) {
     return v;
 }
 
+// shared memory of a cluster: the address of this block's `addr` in block
+// `rank`, loads and stores by such addresses, and the cluster's barrier (with
+// release and acquire)
+__device__ __forceinline__ unsigned cluster_map(unsigned addr, int rank) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+template <class V> __device__ __forceinline__ V ld_cluster(unsigned a) {
+    V v;
+    if constexpr (sizeof(v.x) == 8)
+        asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a));
+    else
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void st_cluster(unsigned a, unsigned long long v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // double-float ("ff") arithmetic on the binary32 pipes.
 //

@@ -50,6 +50,7 @@ namespace hz {
 constexpr int kPsMaxCta = 160;       // CTAs of one system: five per polling lane
 constexpr int kPsMaxWarps = 16;      // warps per CTA, a multiple of 4
 constexpr int kPsMinWarps = 4;
+constexpr int kPsMaxCluster = 16;    // CTAs of one cluster
 constexpr uint64_t kPsStartNs = 10000000000ull;   // the first barrier waits for the launch of all CTAs
 constexpr uint64_t kPsWaitNs = 4000000000ull;
 
@@ -116,6 +117,7 @@ struct PsShared {
     double val[3][kPsMaxWarps * 32];   // per-thread sums (binary32 ones in the first half)
     double scr[3][40];                 // fold scratch of one warp each
     double tot[3];
+    double cl[2][3][kPsMaxCluster];    // sums of the CTAs of a cluster
     int err;
 };
 
@@ -141,15 +143,51 @@ __device__ __forceinline__ R warp_fold(R a, R *buf) {
 // global writes made before it are visible after it (the barriers after the
 // products and F5 publish nothing but sums; a gathered vector is overwritten
 // only after a later barrier with the fence).  False when a wait expired.
-template <class R, int NV, bool kFence, class F>
+// kLive 3: the CTAs are one cluster.  The sums go straight into every CTA's
+// shared memory and the hardware's cluster barrier stands for the lines.
+template <int kLive, class R, int NV, bool kFence, class F>
 __device__ __forceinline__ bool grp_reduce(Grp &g, PsShared &sh, const R (&v)[NV > 0 ? NV : 1], F fin) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     if constexpr (NV > 0) {
 #pragma unroll
         for (int q = 0; q < NV; ++q) reinterpret_cast<R *>(sh.val[q])[threadIdx.x] = v[q];
     }
-    __syncthreads();
     const unsigned long long e = ++g.epoch;
+    if constexpr (kLive == 3) {
+        if constexpr (NV > 0) {
+            R *scr = reinterpret_cast<R *>(sh.scr[warp < NV ? warp : 0]);
+            R a = R(0);
+            __syncthreads();
+            if (warp < NV) {
+                const R *p = reinterpret_cast<const R *>(sh.val[warp]) + lane;
+                for (int w = 0; w < nwarps; w += 4) a += (p[32 * w] + p[32 * w + 32]) + (p[32 * w + 64] + p[32 * w + 96]);
+                a = warp_fold(a, scr);
+                if (lane < g.size) st_cluster(cluster_map(smem_addr(&sh.cl[e & 1][warp][g.rank]), lane), unit_bits(a));
+                __syncwarp();
+            }
+            cluster_barrier();
+            if (warp < NV) {
+                a = lane < g.size ? unit_value<R>((unsigned long long)__double_as_longlong(sh.cl[e & 1][warp][lane])) : R(0);
+                a = warp_fold(a, scr);
+                if (NV > 1) {
+                    if (lane == 0) reinterpret_cast<R *>(sh.tot)[warp] = a;
+                    asm volatile("bar.sync 1, %0;" ::"r"(32 * NV) : "memory");
+                }
+                if (warp == 0) {
+                    R tot[NV];
+                    tot[0] = a;
+#pragma unroll
+                    for (int q = 1; q < NV; ++q) tot[q] = reinterpret_cast<R *>(sh.tot)[q];
+                    fin(tot, lane);
+                }
+            }
+            __syncthreads();
+        } else {
+            cluster_barrier();
+        }
+        return true;
+    }
+    __syncthreads();
     if (warp < (NV > 0 ? NV : 1)) {
         R a = R(0);
         R *scr = reinterpret_cast<R *>(sh.scr[warp]);
@@ -214,10 +252,10 @@ __device__ __forceinline__ bool grp_reduce(Grp &g, PsShared &sh, const R (&v)[NV
     __syncthreads();
     return sh.err == 0;
 }
-template <class R>
+template <int kLive, class R>
 __device__ __forceinline__ bool grp_sync(Grp &g, PsShared &sh) {
     const R v[1] = {R(0)};
-    return grp_reduce<R, 0, true>(g, sh, v, [](R *, int) {});
+    return grp_reduce<kLive, R, 0, true>(g, sh, v, [](R *, int) {});
 }
 
 // component `part` (0 real, 1 imaginary) of a / b, as cdiv: the lanes of a
@@ -270,14 +308,21 @@ struct PsEpi {
     F f;
     template <int N> __device__ void row(int i, V y, Acc (&acc)[N]) const { f(i, y, acc); }
 };
+// how a product gathers a vector: from global memory, or from its part `own`
+// of each CTA's shared memory, `base` being the vector that staged columns address
+template <int kLive, class V>
+__device__ __forceinline__ auto ps_gather(const void *global, const V *own, const V *base) {
+    if constexpr (kLive == 3) return GatherCluster<V>{(unsigned)((const char *)own - (const char *)base)};
+    else return GatherLive<V>{(const V *)global};
+}
 // (wait: the barrier after which x may be gathered; false leaves the product out)
-template <int kLive, class V, int NV, class W, class F>
-__device__ __forceinline__ void ps_product(const MatView<V> &A, const V *x, const Own &o,
+template <int kLive, class V, int NV, class G, class W, class F>
+__device__ __forceinline__ void ps_product(const MatView<V> &A, const G &gx, const Own &o,
                                            typename Ar<V>::Acc (&acc)[NV], W wait, F f) {
     PsEpi<V, NV, F> epi{f};
 #pragma unroll
     for (int j = 0; j < NV; ++j) Ar<V>::acc_zero(acc[j]);
-    slice_rows<V, PsEpi<V, NV, F>, NV, kLive, W>(A, x, epi, acc, o.lo + (int)(threadIdx.x >> 5), (int)(blockDim.x >> 5),
+    slice_rows<V, PsEpi<V, NV, F>, NV, kLive, G, W>(A, gx, epi, acc, o.lo + (int)(threadIdx.x >> 5), (int)(blockDim.x >> 5),
                                                 o.hi, wait);
 }
 
@@ -325,19 +370,19 @@ __device__ bool ps_bicg_loop(const MatView<V> &A, const Ctl &ctl, const Own &o, 
             o.rows([&](int i) {
                 const V q = T::axpy(r[i], beta, T::axmy(p[i], omega, v[i]));
                 p[i] = q;
-                gp[i] = q;
+                if constexpr (kLive != 3) gp[i] = q;
             });
         }
         {   // F2
             typename T::Acc acc[2];
-            ps_product<kLive, V, 2>(A, gp, o, acc, [&]() { return grp_sync<R>(g, sh); },
+            ps_product<kLive, V, 2>(A, ps_gather<kLive>(gp, p, x), o, acc, [&]() { return grp_sync<kLive, R>(g, sh); },
                              [&](int i, V y, auto &a) {
                                  v[i] = y;
                                  T::dotc(a[0], a[1], rh[i], y);
                              });
             if (sh.err) return false;
             const R red[2] = {T::total(acc[0]), T::total(acc[1])};
-            if (!grp_reduce<R, 2, false>(g, sh, red, [&](R(&tot)[2], int lane) {
+            if (!grp_reduce<kLive, R, 2, false>(g, sh, red, [&](R(&tot)[2], int lane) {
                     const auto sig = cmk(tot[0], tot[1]);
                     const R q = cdiv_part(st.rho, sig, lane & 1);
                     if (lane == 0 && cis_zero(sig)) { st.status = HZ_BREAKDOWN; st.done = 1; }
@@ -355,16 +400,16 @@ __device__ bool ps_bicg_loop(const MatView<V> &A, const Ctl &ctl, const Own &o, 
             o.rows([&](int i) {
                 const V q = T::axmy(r[i], alpha, v[i]);
                 s[i] = q;
-                gs[i] = q;
+                if constexpr (kLive != 3) gs[i] = q;
                 T::nrm2(acc[0], q);
             });
             ssum[0] = T::total(acc[0]);
         }
         typename T::Acc acc4[3];
         ps_product<kLive, V, 3>(   // F4, behind the barrier with ||s||^2
-            A, gs, o, acc4,
+            A, ps_gather<kLive>(gs, s, x), o, acc4,
             [&]() {
-                return grp_reduce<R, 1, true>(g, sh, ssum, [&](R(&tot)[1], int lane) {
+                return grp_reduce<kLive, R, 1, true>(g, sh, ssum, [&](R(&tot)[1], int lane) {
                            const double ss = (double)tot[0];
                            if (lane != 0 || ss > st.thr) {
                                if (lane == 0 && !finite_d(ss)) {
@@ -395,7 +440,7 @@ __device__ bool ps_bicg_loop(const MatView<V> &A, const Ctl &ctl, const Own &o, 
         }
         {
             const R red[3] = {T::total(acc4[0]), T::total(acc4[1]), T::total(acc4[2])};
-            if (!grp_reduce<R, 3, false>(g, sh, red, [&](R(&tot)[3], int lane) {
+            if (!grp_reduce<kLive, R, 3, false>(g, sh, red, [&](R(&tot)[3], int lane) {
                     const R q = (lane & 1 ? tot[1] : tot[0]) / tot[2];
                     if (lane == 0 && tot[2] == R(0)) { st.status = HZ_BREAKDOWN; st.done = 1; }
                     if (lane == 0) st.omega.x = q;
@@ -426,7 +471,7 @@ __device__ bool ps_bicg_loop(const MatView<V> &A, const Ctl &ctl, const Own &o, 
                 T::nrm2(acc[2], ri);
             });
             const R red[3] = {T::total(acc[0]), T::total(acc[1]), T::total(acc[2])};
-            if (!grp_reduce<R, 3, false>(g, sh, red, [&](R(&tot)[3], int lane) {
+            if (!grp_reduce<kLive, R, 3, false>(g, sh, red, [&](R(&tot)[3], int lane) {
                     const auto rn = cmk(tot[0], tot[1]);
                     const R bq = cmul_part(rn, st.fac, lane & 1);
                     if (lane == 1) st.beta.y = bq;
@@ -498,11 +543,11 @@ __device__ void ps_finish(const PsSys &S, const MatView<double2> &A, const Own &
     const Ctl &c = S.ctl;
     o.rows([&](int i) { S.x[i] = x[i]; });
     double acc[1];
-    ps_product<kLive, double2, 1>(A, S.x, o, acc, [&]() { return grp_sync<double>(g, sh); },
+    ps_product<kLive, double2, 1>(A, ps_gather<kLive>(S.x, x, x), o, acc, [&]() { return grp_sync<kLive, double>(g, sh); },
                                   [&](int i, double2 y, auto &a) { Ar<double2>::nrm2(a[0], csub(c.b[i], y)); });
     if (sh.err) return;
     const bool lead = g.rank == 0;
-    if (!grp_reduce<double, 1, true>(g, sh, acc, [&](double(&tot)[1], int lane) {
+    if (!grp_reduce<kLive, double, 1, true>(g, sh, acc, [&](double(&tot)[1], int lane) {
             if (!lead || lane != 0) return;
             S.info->iters = st.iter;
             S.info->status = st.status;
@@ -546,15 +591,21 @@ __device__ __forceinline__ const PsSys *ps_setup(const PsSys *sys, int nsys, Own
 
 extern __shared__ __align__(16) unsigned char ps_smem[];
 
+// rows of a vector's part in shared memory (the same in every CTA of a cluster)
+template <int kLive>
+__device__ __forceinline__ int ps_rows(const Own &o, const Grp &g, int nsl) {
+    return 32 * (kLive == 3 ? (nsl + g.size - 1) / g.size : o.hi - o.lo);
+}
+
 // The own slices of the stream in shared memory behind `at` (kLive 2), where
 // they and the Krylov vectors fit there: a view that reads them from there.
 // Between a barrier and its gathers there is then no other latency, and
 // neither the columns nor the values are read through L2 in every pass (the
 // fences of the barriers empty L1).
 template <int kLive, class V>
-__device__ __forceinline__ MatView<V> ps_stage(const MatView<V> &A, const Own &o, void *at) {
+__device__ __forceinline__ MatView<V> ps_stage(const MatView<V> &A, const Own &o, const Grp &g, void *at) {
     MatView<V> M = A;
-    if constexpr (kLive == 2) {
+    if constexpr (kLive >= 2) {
         const int b0 = A.sl_base[o.lo], cnt = 32 * (A.sl_base[o.hi] - b0), ns = o.hi - o.lo;
         const size_t off = (size_t)32 * b0;
         unsigned long long *mask = (unsigned long long *)at;
@@ -577,7 +628,15 @@ __device__ __forceinline__ MatView<V> ps_stage(const MatView<V> &A, const Own &o
             M.sl_val32 = v - off;
         }
         int *col = (int *)q, *base = col + cnt;
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) col[i] = A.sl_col[off + i];
+        for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+            int c = A.sl_col[off + i];
+            if (kLive == 3 && c >= 0) {   // the address of the first vector's entry c in the CTA that owns it
+                const int r = (int)(((int64_t)((c >> 5) + 1) * g.size - 1) / A.nsl);
+                const int lo = (int)((int64_t)A.nsl * r / g.size);
+                c = (int)cluster_map(smem_addr(ps_smem) + (unsigned)(c - 32 * lo) * (unsigned)sizeof(V), r);
+            }
+            col[i] = c;
+        }
         for (int i = threadIdx.x; i <= ns; i += blockDim.x) base[i] = A.sl_base[o.lo + i];
         M.sl_col = col - off;
         M.sl_base = base - o.lo;
@@ -595,19 +654,19 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_bicg(const PsSys *sy
     Grp g;
     const PsSys &S = *ps_setup(sys, nsys, o, g, sh);
     const Ctl &ctl = S.ctl;
-    const int m = (o.hi - o.lo) * 32;
+    const int m = ps_rows<kLive>(o, g, S.A.nsl);
     // vectors indexed by row: each points 32 lo entries before its part
     double2 *base = reinterpret_cast<double2 *>(ps_smem) - 32 * o.lo;
     double2 *x = base, *r = base + m, *rh = base + 2 * m, *p = base + 3 * m, *v = base + 4 * m, *s = base + 5 * m,
             *t = base + 6 * m;
-    const MatView<double2> M = ps_stage<kLive>(S.A, o, reinterpret_cast<double2 *>(ps_smem) + 7 * m);
+    const MatView<double2> M = ps_stage<kLive>(S.A, o, g, reinterpret_cast<double2 *>(ps_smem) + 7 * m);
     if (threadIdx.x == 0) {
         st.iter = ctl.restart ? S.info->iters : 0;
         st.zero_x = 0;
     }
     ps_start_x(S, o, x);
     double acc[2];
-    ps_product<kLive, double2, 2>(M, S.x, o, acc, [&]() { return grp_sync<double>(g, sh); },
+    ps_product<kLive, double2, 2>(M, ps_gather<kLive>(S.x, x, x), o, acc, [&]() { return grp_sync<kLive, double>(g, sh); },
                            [&](int i, double2 y, auto &a) {
                                const double2 bi = ctl.b[i], ri = csub(bi, y);
                                r[i] = ri;
@@ -618,7 +677,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_bicg(const PsSys *sy
                                Ar<double2>::nrm2(a[1], bi);
                            });
     if (sh.err) return;
-    if (!grp_reduce<double, 2, true>(g, sh, acc, [&](double(&tot)[2], int lane) {
+    if (!grp_reduce<kLive, double, 2, true>(g, sh, acc, [&](double(&tot)[2], int lane) {
             if (lane == 0) ps_start_state(ctl, st, tot[0], tot[1], g.rank == 0);
         }))
         return;
@@ -646,11 +705,11 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_mixed(const PsSys *s
     const PsSys &S = *ps_setup(sys, nsys, o, g, sh);
     const Ctl &ctl = S.ctl;
     const bool lead = g.rank == 0;
-    const int m = (o.hi - o.lo) * 32;
+    const int m = ps_rows<kLive>(o, g, S.A.nsl);
     float2 *base = reinterpret_cast<float2 *>(ps_smem) - 32 * o.lo;
     float2 *d = base, *r = base + m, *rh = base + 2 * m, *p = base + 3 * m, *v = base + 4 * m, *s = base + 5 * m,
            *t = base + 6 * m;
-    const MatView<float2> M = ps_stage<kLive>(S.A32, o, reinterpret_cast<float2 *>(ps_smem) + 7 * m);
+    const MatView<float2> M = ps_stage<kLive>(S.A32, o, g, reinterpret_cast<float2 *>(ps_smem) + 7 * m);
     if (threadIdx.x == 0) {
         ou.outer = 0; ou.done = 0; ou.status = HZ_NOT_CONVERGED; ou.zero_x = 0;
         ou.best = INFINITY; ou.save = 0; ou.use_best = 0; ou.total = 0;
@@ -658,7 +717,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_mixed(const PsSys *s
     ps_start_x(S, o, nullptr);
     for (int run = 0; run <= ctl.max_outer; ++run) {
         double acc[3];
-        ps_product<1, double2, 3>(S.A, S.x, o, acc, [&]() { return grp_sync<double>(g, sh); },
+        ps_product<1, double2, 3>(S.A, GatherLive<double2>{S.x}, o, acc, [&]() { return grp_sync<kLive, double>(g, sh); },
                                [&](int i, double2 y, auto &a) {
                                    const double2 bi = ctl.b[i], ri = csub(bi, y);
                                    const float2 r32 = to_c64(ri), z = make_float2(0.f, 0.f);
@@ -672,7 +731,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_mixed(const PsSys *s
                                    Ar<double2>::nrm2(a[2], to_c128(r32));
                                });
         if (sh.err) return;
-        if (!grp_reduce<double, 3, true>(g, sh, acc, [&](double(&tot)[3], int lane) {
+        if (!grp_reduce<kLive, double, 3, true>(g, sh, acc, [&](double(&tot)[3], int lane) {
                 if (lane != 0) return;
                 const double nb = sqrt(tot[1]);
                 ou.done = 1;
@@ -744,21 +803,31 @@ struct PsTq {
     int m, stop, pend;
 };
 
-// one half step from W (all lanes of a warp; lanes 0..5 divide: coef re/im,
-// c^2, tau^2 factor, theta^2, and beta = rho1 / rho for the second half step)
-__device__ __forceinline__ void ps_tq_half(PsTq &t, double2 alpha, double W, int lane) {
+// One half step from W, and beta = rho1 / rho for the second one, by all lanes
+// of a warp with one division each: lanes 0, 1 coef = theta^2 eta / alpha,
+// 2 c^2, 3 the factor of tau^2, 4 the new theta^2, 5, 6 beta.
+__device__ __forceinline__ void ps_tq_half(PsTq &t, double2 alpha, double W, double2 rho1, double2 rho, double2 &beta,
+                                           int lane) {
+    const bool first = lane < 2;
     const double2 te = make_double2(t.th2 * t.eta.x, t.th2 * t.eta.y);
-    const double tau2 = t.tau2, s = tau2 + W, aa = alpha.x * alpha.x + alpha.y * alpha.y;
-    double num, den;
-    switch (lane) {
-        case 0: num = te.x * alpha.x + te.y * alpha.y; den = aa; break;
-        case 1: num = te.y * alpha.x - te.x * alpha.y; den = aa; break;
-        case 2: num = tau2; den = s; break;
-        case 3: num = W; den = s; break;
-        default: num = W; den = tau2; break;
-    }
-    const double q = num / den;
+    const double2 a = first ? te : rho1;
+    double2 b = first ? alpha : rho;
+    const int part = first ? lane : lane == 6;
+    const double tau2 = t.tau2, s = tau2 + W;
+    // a / b as cdiv_part, up to the division
+    const int e = max(__double2hiint(b.x) & 0x7ff00000, __double2hiint(b.y) & 0x7ff00000) >> 20;
+    const double sc = __hiloint2double((2046 - min(2045, max(1, e))) << 20, 0);
+    b.x *= sc;
+    b.y *= sc;
+    const double d = b.x * b.x + b.y * b.y;
+    const double y0 = part ? b.x : b.y, y1 = part ? -b.y : b.x;
+    const double n = a.y * y0 + a.x * y1;
+    const bool mid = lane >= 2 && lane < 5;
+    const double num = mid ? (lane == 2 ? tau2 : W) : n, den = mid ? (lane == 4 ? tau2 : s) : d;
+    const double q = num / den * (mid ? 1.0 : sc);
     if (lane < 5) t.q[lane] = q;
+    if (lane == 5) beta.x = q;
+    if (lane == 6) beta.y = q;
     __syncwarp();
     if (lane == 0) {
         const bool z = tau2 == 0.0;
@@ -783,12 +852,12 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
     const PsSys &S = *ps_setup(sys, nsys, o, g, sh);
     const Ctl &ctl = S.ctl;
     const bool lead = g.rank == 0, hist = lead && ctl.hist;
-    const int m = (o.hi - o.lo) * 32;
+    const int m = ps_rows<kLive>(o, g, S.A.nsl);
     double2 *base = reinterpret_cast<double2 *>(ps_smem) - 32 * o.lo;
     double2 *x = base, *w = base + m, *u1 = base + 2 * m, *u2 = base + 3 * m, *v = base + 4 * m, *d = base + 5 * m,
             *au1 = base + 6 * m, *au = base + 7 * m, *rh = base + 8 * m;
     double2 *gu1 = (double2 *)S.g0, *gu2 = (double2 *)S.g1;
-    const MatView<double2> M = ps_stage<kLive>(S.A, o, reinterpret_cast<double2 *>(ps_smem) + 9 * m);
+    const MatView<double2> M = ps_stage<kLive>(S.A, o, g, reinterpret_cast<double2 *>(ps_smem) + 9 * m);
     if (threadIdx.x == 0) {
         st.iter = ctl.restart ? S.info->iters : 0;
         st.zero_x = 0;
@@ -796,7 +865,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
     ps_start_x(S, o, x);
     {
         double acc[2];
-        ps_product<kLive, double2, 2>(M, S.x, o, acc, [&]() { return grp_sync<double>(g, sh); },
+        ps_product<kLive, double2, 2>(M, ps_gather<kLive>(S.x, x, x), o, acc, [&]() { return grp_sync<kLive, double>(g, sh); },
                                [&](int i, double2 y, auto &a) {
                                    const double2 bi = ctl.b[i], ri = csub(bi, y), z = make_double2(0.0, 0.0);
                                    w[i] = ri;
@@ -809,7 +878,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
                                    A::nrm2(a[1], bi);
                                });
         if (sh.err) return;
-        if (!grp_reduce<double, 2, true>(g, sh, acc, [&](double(&tot)[2], int lane) {
+        if (!grp_reduce<kLive, double, 2, true>(g, sh, acc, [&](double(&tot)[2], int lane) {
                 if (lane != 0) return;
                 q.tau2 = tot[0];
                 q.th2 = 0.0;
@@ -826,7 +895,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
     while (!st.done) {
         {   // Q4: au1 = A u1, v += au1, <r^, v>, ||v||^2 -> alpha
             double acc[3];
-            ps_product<kLive, double2, 3>(M, gu1, o, acc, [&]() { return first || grp_sync<double>(g, sh); },
+            ps_product<kLive, double2, 3>(M, ps_gather<kLive>(gu1, u1, x), o, acc, [&]() { return first || grp_sync<kLive, double>(g, sh); },
                                    [&](int i, double2 y, auto &a) {
                                        au1[i] = y;
                                        const double2 vi = A::add(y, v[i]);
@@ -836,7 +905,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
                                    });
             first = false;
             if (sh.err) return;
-            if (!grp_reduce<double, 3, false>(g, sh, acc, [&](double(&tot)[3], int lane) {
+            if (!grp_reduce<kLive, double, 3, false>(g, sh, acc, [&](double(&tot)[3], int lane) {
                     const double2 sig = make_double2(tot[0], tot[1]);
                     const double c = cdiv_part(st.rho, sig, lane & 1);
                     const bool brk = cis_zero(st.rho) || cis_zero(sig);
@@ -867,7 +936,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
             }
             const double2 u = A::axmy(u1i, alpha, vi);
             u2[i] = u;
-            gu2[i] = u;
+            if constexpr (kLive != 3) gu2[i] = u;
             wi = A::axmy(wi, alpha, ai);
             w[i] = wi;
             A::nrm2(ww[0], wi);
@@ -876,9 +945,9 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
         // Q2, behind the barrier with ||w||^2: au = A u2; d, x and w
         double2 coef, eta;
         ps_product<kLive, double2, 3>(
-            M, gu2, o, acc,
+            M, ps_gather<kLive>(gu2, u2, x), o, acc,
             [&]() {
-                const bool ok = grp_reduce<double, 1, true>(g, sh, ww, [&](double(&tot)[1], int lane) {
+                const bool ok = grp_reduce<kLive, double, 1, true>(g, sh, ww, [&](double(&tot)[1], int lane) {
                     if (pend && lane == 0) {
                         q.pend = 0;
                         q.tau2 *= kTqShrink * kTqShrink;
@@ -886,7 +955,8 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
                         q.xs /= kTqShrink;
                     }
                     __syncwarp();
-                    ps_tq_half(q, alpha, tot[0], lane);
+                    double2 none;
+                    ps_tq_half(q, alpha, tot[0], alpha, alpha, none, lane);
                 });
                 coef = q.coef;
                 eta = q.etax;
@@ -903,14 +973,10 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
                 A::dotc(a[1], a[2], rh[i], wi);
             });
         if (sh.err) return;
-        if (!grp_reduce<double, 3, false>(g, sh, acc, [&](double(&tot)[3], int lane) {
-                ps_tq_half(q, alpha, tot[0], lane);
+        if (!grp_reduce<kLive, double, 3, false>(g, sh, acc, [&](double(&tot)[3], int lane) {
                 const double2 rho1 = make_double2(tot[1], tot[2]);
-                const double b = cdiv_part(rho1, st.rho, lane & 1);
-                __syncwarp();
-                if (lane == 1) st.beta.y = b;
+                ps_tq_half(q, alpha, tot[0], rho1, st.rho, st.beta, lane);
                 if (lane != 0) return;
-                st.beta.x = b;
                 const int it = st.iter + 1;
                 st.iter = it;
                 st.rho = rho1;
@@ -934,7 +1000,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
             if (!stop) {
                 const double2 u = A::axpy(w[i], beta, ui);
                 u1[i] = u;
-                gu1[i] = u;
+                if constexpr (kLive != 3) gu1[i] = u;
                 v[i] = A::axpy(A::zero(), beta, A::axpy(au[i], beta, v[i]));
             }
         });
@@ -946,16 +1012,16 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
 // ---------------------------------------------------------------------------
 // host side
 struct PsMethod {
-    void *kern[2];   // the matrix through L2; staged in shared memory
+    void *kern[3];   // the matrix through L2; staged in shared memory; and one cluster
     int vecs;        // Krylov vectors in shared memory
     int elem;        // bytes per element
     int slot;        // bytes per slot of the staged stream
 };
 static PsMethod ps_method(PsKind k) {
     switch (k) {
-        case PS_BICG: return {{(void *)k_ps_bicg<1>, (void *)k_ps_bicg<2>}, 7, 16, 20};
-        case PS_MIXED: return {{(void *)k_ps_mixed<1>, (void *)k_ps_mixed<2>}, 7, 8, 12};
-        default: return {{(void *)k_ps_tfqmr<1>, (void *)k_ps_tfqmr<2>}, 9, 16, 20};
+        case PS_BICG: return {{(void *)k_ps_bicg<1>, (void *)k_ps_bicg<2>, (void *)k_ps_bicg<3>}, 7, 16, 20};
+        case PS_MIXED: return {{(void *)k_ps_mixed<1>, (void *)k_ps_mixed<2>, (void *)k_ps_mixed<3>}, 7, 8, 12};
+        default: return {{(void *)k_ps_tfqmr<1>, (void *)k_ps_tfqmr<2>, (void *)k_ps_tfqmr<3>}, 9, 16, 20};
     }
 }
 constexpr int kPsSmem = 212 * 1024;   // dynamic shared memory of a CTA at most (227 KB less the static part)
@@ -1012,6 +1078,52 @@ static cudaError_t ps_launch(PsKind kind, hz_mat *const *A, const PsSys *h, int 
     if (e != cudaSuccess) return e;
     void *args[] = {&dsys, &ns};
     return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(32 * warps), args, st ? staged : plain, s);
+}
+
+// One cluster for the smallest systems: on 16 SMs the gathers and sums go
+// through the cluster's shared memory, a pass waits for no L2 latency, but has
+// a tenth of the binary64 pipes.  us per iteration, cluster / all SMs:
+//   unknowns           512          1.7k         4.1k         5.8k         8k          13.8k
+//   BiCGStab    15.4 / 21.0  16.0 / 21.2  17.9 / 22.8  20.7 / 23.9  24.1 / 23.4  24.6* / 24.5
+//   TFQMR       15.5 / 19.3  15.1 / 20.4  17.6 / 21.5  20.8 / 22.9  24.4 / 22.8
+//   mixed        7.0 /  9.7   6.7 / 10.5   7.3 / 11.9   7.3 / 11.9   7.9 / 12.3   9.0 / 12.5
+// (* does not fit).  So up to 12 slices per CTA in binary64, 32 (as many as
+// always fit with rows of 15) in the mixed method, whose passes run on the
+// binary32 pipes.  The CTAs (0: not this way) and their shared memory:
+static int ps_cluster(const hz_mat *A, PsKind kind, size_t *smem) {
+    const PsMethod m = ps_method(kind);
+    int c = 1;
+    while (c < kPsMaxCluster && c < A->nsl) c *= 2;
+    const int per = (A->nsl + c - 1) / c;
+    if (per > (kind == PS_MIXED ? 32 : 12)) return 0;
+    int steps = 0;
+    for (int r = 0; r < c; ++r)
+        steps = std::max(steps, A->sl_base_h[(int64_t)A->nsl * (r + 1) / c] - A->sl_base_h[(int64_t)A->nsl * r / c]);
+    *smem = (size_t)per * 32 * m.vecs * m.elem + (size_t)32 * steps * m.slot + (size_t)per * 12 + 4;
+    return *smem <= (size_t)kPsSmem ? c : 0;
+}
+
+static cudaError_t ps_launch_cluster(PsKind kind, int ctas, int slices, size_t smem, PsSys *dsys, cudaStream_t s) {
+    void *kern = ps_method(kind).kern[2];
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPsSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    const int warps = std::min(kPsMaxWarps, std::max(kPsMinWarps, (slices + 3) / 4 * 4));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(32 * warps);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int ns = 1;
+    void *args[] = {&dsys, &ns};
+    return cudaLaunchKernelExC(&cfg, kern, args);
 }
 
 struct PsSolver {
@@ -1084,12 +1196,15 @@ hz_status ps_solve(hz_mat *A, PsKind kind, const Ctl &c, Info *out, int *restart
     h.ctl = c;
     h.info = S->dinfo; h.lines = S->lines; h.err = S->err;
     h.cta0 = 0;
-    h.ncta = ps_ctas(A, d.num_sms);
+    size_t smem = 0;
+    const int cl = ps_cluster(A, kind, &smem);
+    h.ncta = cl ? cl : ps_ctas(A, d.num_sms);
     *restarts = 0;
     for (int run = 0;; ++run) {
         HZ_CUDA(cudaMemcpyAsync(S->dsys, &h, sizeof(PsSys), cudaMemcpyHostToDevice, s));
         HZ_CUDA(cudaMemsetAsync(S->lines, 0, kPsErrOff + sizeof(int), s));
-        HZ_CUDA(ps_launch(kind, &A, &h, 1, S->dsys, s));
+        HZ_CUDA(cl ? ps_launch_cluster(kind, cl, (A->nsl + cl - 1) / cl, smem, S->dsys, s)
+                   : ps_launch(kind, &A, &h, 1, S->dsys, s));
         HZ_CUDA(cudaMemcpyAsync(&S->hback->info, S->dinfo, sizeof(Info), cudaMemcpyDeviceToHost, s));
         HZ_CUDA(cudaMemcpyAsync(&S->hback->err, S->err, sizeof(int), cudaMemcpyDeviceToHost, s));
         HZ_CUDA(cudaStreamSynchronize(s));

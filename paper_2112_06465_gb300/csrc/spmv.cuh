@@ -1102,11 +1102,24 @@ struct NoWait {
 };
 // kLive: 1: x was written by other blocks of the running kernel (read it
 // through L2), and the matrix is read again every iteration (let L1 keep it);
-// 2: and the slices s0 .. send of the stream are in shared memory.
+// 2: and the slices s0 .. send of the stream are in shared memory; 3: and
+// their columns are shared-memory addresses in a cluster.  gx(c): x at column c.
 // wait() runs once on every thread after the first columns are requested and
 // before x is read; the rows are left out if it returns false.
-template <class V, class Epi, int NV, int kLive = 0, class Wait = NoWait>
-__device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, const Epi &epi,
+template <class V> struct GatherConst {   // x is not written while the kernel runs
+    const V *x;
+    __device__ V operator()(int c) const { return __ldg(x + c); }
+};
+template <class V> struct GatherLive {
+    const V *x;
+    __device__ V operator()(int c) const { return ld_live(x + c); }
+};
+template <class V> struct GatherCluster {   // off: bytes from the vector that the columns address
+    unsigned off;
+    __device__ V operator()(int c) const { return ld_cluster<V>((unsigned)c + off); }
+};
+template <class V, class Epi, int NV, int kLive = 0, class Gather = GatherConst<V>, class Wait = NoWait>
+__device__ __forceinline__ void slice_rows(const MatView<V> &A, const Gather &gx, const Epi &epi,
                                            typename Epi::Acc (&acc)[NV], int s0, int step, int send,
                                            Wait wait = Wait{}) {
     constexpr bool kD = std::is_same<V, double2>::value;
@@ -1120,7 +1133,7 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, cons
     auto meta = [&](int s) {
         Sl q{s, 0, 0, 0ull};
         if (s < send) {
-            if constexpr (kLive == 2) {
+            if constexpr (kLive >= 2) {
                 q.b = A.sl_base[s];
                 q.w = A.sl_base[s + 1] - q.b;
                 if constexpr (kD) q.m = A.sl_mask[s];
@@ -1133,14 +1146,11 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, cons
         return q;
     };
     auto ldm = [&](const auto *p) {
-        if constexpr (kLive == 2) return *p;
+        if constexpr (kLive >= 2) return *p;
         else if constexpr (kLive == 1) return __ldg(p);
         else return ld_stream(p, pol);
     };
-    auto ldx = [&](const V *p) {
-        if constexpr (kLive != 0) return ld_live(p);
-        else return __ldg(p);
-    };
+    auto has = [](int c) { return kLive == 3 ? c != -1 : c >= 0; };
     // the column stream runs one group ahead, across slices
     auto cols = [&](const Sl &q, int u0, int (&c)[G]) {
         const int *p = A.sl_col + (size_t)32 * (q.b + u0) + lane;
@@ -1179,7 +1189,7 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const V *x, cons
             if (u0 + G < w) cols(cur, u0 + G, cn);
             else cols(nxt, 0, cn);
 #pragma unroll
-            for (int u = 0; u < G; ++u) v[u] = c[u] >= 0 ? ldx(x + c[u]) : czero<V>();
+            for (int u = 0; u < G; ++u) v[u] = has(c[u]) ? gx(c[u]) : czero<V>();
             const int left = w - u0;
             if (left > G) {
                 if (kD && !(mg & ((1u << G) - 1u))) slice_group<G, kD, false>(y, y2, a, v, bad_re, bad_im);
@@ -1248,7 +1258,7 @@ __global__ void __launch_bounds__(kFlatThreads, kSlMinBlocks<V>) k_spmv_sl(MatVi
 #pragma unroll
     for (int j = 0; j < NV; ++j) Epi::zero(acc[j]);
     const int wpc = blockDim.x >> 5;
-    slice_rows<V, Epi, NV>(A, x, epi, acc, blockIdx.x * wpc + (threadIdx.x >> 5), gridDim.x * wpc, A.nsl);
+    slice_rows<V, Epi, NV>(A, GatherConst<V>{x}, epi, acc, blockIdx.x * wpc + (threadIdx.x >> 5), gridDim.x * wpc, A.nsl);
     if constexpr (Epi::NV > 0) spmv_reduce<Epi, NV>(epi, acc, red);
 }
 

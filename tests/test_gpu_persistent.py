@@ -48,9 +48,10 @@ def vec(n, seed):
 
 METHODS = [dict(method="bicgstab"), dict(method="tfqmr"), dict(mode="mixed"),
            dict(method="bicgstab", precond="jacobi"), dict(method="tfqmr", precond="jacobi")]
-# 152 x 32 = 4864 rows give every SM one slice; 60 x 4864 is the most that
+# 12 x 512 = 6144 rows are the most of a binary64 cluster, 32 x 512 of a mixed
+# one; 152 x 32 = 4864 rows give every SM one slice; 60 x 4864 is the most that
 # BiCGStab in binary64 holds on chip, 47 x 4864 TFQMR
-SIZES = [1, 2, 31, 33, 1000, 4864, 4865, 20011, 100003, 47 * 4864, 60 * 4864, 60 * 4864 + 1]
+SIZES = [1, 2, 31, 33, 1000, 4864, 4865, 6144, 6145, 16384, 16385, 20011, 100003, 47 * 4864, 60 * 4864, 60 * 4864 + 1]
 
 
 @pytest.mark.parametrize("n", SIZES)
