@@ -117,6 +117,6 @@ def load():
 
 def check(status: int, allow=(HZ_OK,)):
     """Raise HzError unless status is in `allow`; returns the status."""
-    if status not in allow:
+    if status != HZ_OK and status not in allow:   # (HZ_OK is in every list)
         raise HzError(status, load().hz_last_error().decode(errors="replace"))
     return status

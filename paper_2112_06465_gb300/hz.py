@@ -20,12 +20,19 @@ from ._lib import (HZ_FLAG_AUTOTUNE, HZ_FLAG_C64, HZ_FLAG_SELL, HZ_FLAG_VALIDATE
 _L = _lib.load()
 
 
+# The addresses go to ctypes as plain integers (the argument types make void
+# pointers of them) and the current stream comes as its raw handle: on short
+# vectors a BLAS-1 call is mostly this code, and stream and pointer objects
+# were a good part of it.
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(_device())
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _vec(t, dtype=torch.complex128, name="vector"):
@@ -142,7 +149,7 @@ def _pair(x, y):
 def zdotc(x, y, out=None):
     """sum conj(x_i) y_i, returned as a 1-element device tensor."""
     x, y = _pair(x, y)
-    out = torch.empty(1, dtype=torch.complex128, device=x.device) if out is None else out
+    out = x.new_empty(1) if out is None else out
     check(_L.hz_zdotc(x.numel(), _ptr(x), _ptr(y), _ptr(out), _stream()))
     return out
 
@@ -150,7 +157,7 @@ def zdotc(x, y, out=None):
 def zdotu(x, y, out=None):
     """sum x_i y_i, returned as a 1-element device tensor."""
     x, y = _pair(x, y)
-    out = torch.empty(1, dtype=torch.complex128, device=x.device) if out is None else out
+    out = x.new_empty(1) if out is None else out
     check(_L.hz_zdotu(x.numel(), _ptr(x), _ptr(y), _ptr(out), _stream()))
     return out
 
@@ -158,14 +165,14 @@ def zdotu(x, y, out=None):
 def dznrm2(x, out=None):
     """sqrt(sum |x_i|^2), returned as a 1-element float64 device tensor."""
     x = _vec(x, name="x")
-    out = torch.empty(1, dtype=torch.float64, device=x.device) if out is None else out
+    out = x.new_empty(1, dtype=torch.float64) if out is None else out
     check(_L.hz_dznrm2(x.numel(), _ptr(x), _ptr(out), _stream()))
     return out
 
 
 def _scalar(alpha, device):
     if isinstance(alpha, torch.Tensor):
-        return _vec(alpha.reshape(1), name="alpha")
+        return _vec(alpha if alpha.dim() == 1 and alpha.numel() == 1 else alpha.reshape(1), name="alpha")
     return torch.tensor([complex(alpha)], dtype=torch.complex128, device=device)
 
 
