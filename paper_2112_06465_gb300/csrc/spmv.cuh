@@ -1037,7 +1037,8 @@ __device__ __forceinline__ void flat_rows_d64(const MatView<double2> &A, const d
 // length of the last group are separate code reached by branches.
 //
 // Measured against the lane runs and, in complex64, the product slab:
-//   618 k rows of 15, real but for the ends   49.5 -> 42.7 us
+//   618 k rows of 15, real but for the ends   49.5 -> 42.7 us (40.8 us with
+//   real steps for real diagonals)
 //   672 k rows of 27, every value complex      209 -> 137 us (at the pipe's
 //   rate for its 72.6 M multiply-adds)
 //   complex64, 618 k rows of 15               23.4 -> 20.6 us
@@ -1059,8 +1060,8 @@ __device__ __forceinline__ void watch_nonfinite(unsigned &bad, double v) {
 
 // One group of N steps into (y, y2): even and odd steps in two chains.  In
 // the final group of a slice the last step is the diagonal's: it is added
-// to the sum of both chains, as a complex step.
-template <int N, bool kReal, bool kFinal, class V, int G>
+// to the sum of both chains, as a complex step or (kRealDiag) a real one.
+template <int N, bool kReal, bool kFinal, bool kRealDiag, class V, int G>
 __device__ __forceinline__ void slice_group(V &y, V &y2, const V (&a)[G], const V (&v)[G], unsigned &bad_re,
                                             unsigned &bad_im) {
     constexpr int M = kFinal ? N - 1 : N;
@@ -1078,22 +1079,29 @@ __device__ __forceinline__ void slice_group(V &y, V &y2, const V (&a)[G], const 
     }
     if constexpr (kFinal) {
         y = cadd(y, y2);
-        cmac(y, a[N - 1], v[N - 1]);
+        if constexpr (kRealDiag) {
+            y.x = fma(a[N - 1].x, v[N - 1].x, y.x);
+            y.y = fma(a[N - 1].x, v[N - 1].y, y.y);
+            watch_nonfinite(bad_re, v[N - 1].y);
+            watch_nonfinite(bad_im, v[N - 1].x);
+        } else {
+            cmac(y, a[N - 1], v[N - 1]);
+        }
     }
 }
-template <bool kReal, class V, int G>
+template <bool kReal, bool kRealDiag, class V, int G>
 __device__ __forceinline__ void slice_final(int n, V &y, V &y2, const V (&a)[G], const V (&v)[G], unsigned &bad_re,
                                             unsigned &bad_im) {
     static_assert(G == 8, "one case per length");
     switch (n) {
-        case 1: slice_group<1, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
-        case 2: slice_group<2, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
-        case 3: slice_group<3, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
-        case 4: slice_group<4, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
-        case 5: slice_group<5, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
-        case 6: slice_group<6, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
-        case 7: slice_group<7, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
-        default: slice_group<8, kReal, true>(y, y2, a, v, bad_re, bad_im); break;
+        case 1: slice_group<1, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
+        case 2: slice_group<2, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
+        case 3: slice_group<3, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
+        case 4: slice_group<4, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
+        case 5: slice_group<5, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
+        case 6: slice_group<6, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
+        case 7: slice_group<7, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
+        default: slice_group<8, kReal, true, kRealDiag>(y, y2, a, v, bad_re, bad_im); break;
     }
 }
 
@@ -1192,11 +1200,14 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const Gather &gx
             for (int u = 0; u < G; ++u) v[u] = has(c[u]) ? gx(c[u]) : czero<V>();
             const int left = w - u0;
             if (left > G) {
-                if (kD && !(mg & ((1u << G) - 1u))) slice_group<G, kD, false>(y, y2, a, v, bad_re, bad_im);
-                else slice_group<G, false, false>(y, y2, a, v, bad_re, bad_im);
+                if (kD && !(mg & ((1u << G) - 1u))) slice_group<G, kD, false, false>(y, y2, a, v, bad_re, bad_im);
+                else slice_group<G, false, false, false>(y, y2, a, v, bad_re, bad_im);
             } else {
-                if (kD && !(mg & ((1u << (left - 1)) - 1u))) slice_final<kD>(left, y, y2, a, v, bad_re, bad_im);
-                else slice_final<false>(left, y, y2, a, v, bad_re, bad_im);
+                if (kLive == 0 && kD && !(mg & ((1u << left) - 1u)))
+                    slice_final<kD, kD>(left, y, y2, a, v, bad_re, bad_im);
+                else if (kD && !(mg & ((1u << (left - 1)) - 1u)))
+                    slice_final<kD, false>(left, y, y2, a, v, bad_re, bad_im);
+                else slice_final<false, false>(left, y, y2, a, v, bad_re, bad_im);
             }
         }
         if (w == 0) cols(nxt, 0, cn);
