@@ -135,8 +135,12 @@ enum {
                                 real part), so every load is coalesced, and the imaginary parts
                                 stored only for groups of steps that have a nonzero one (a group
                                 without is known to be real before its loads; the same sums as
-                                HZ_SPMV_FLAT64).  Device memory: 20 bytes per slot, about nnz
-                                slots.  The default without HZ_FLAG_FF */
+                                HZ_SPMV_FLAT64).  Where neighbouring rows have nearly equal
+                                lengths the copy holds one row per lane instead, the diagonal
+                                entry last (another order of the sums within the same error
+                                bound; the few rows far longer than the others are read from
+                                the caller's arrays).  Device memory: 20 bytes per slot, about
+                                nnz slots.  The default without HZ_FLAG_FF */
 };
 
 typedef struct {
@@ -352,8 +356,11 @@ HZ_API hz_status hz_zsolve_opts(hz_mat *A, const hz_z *d_b, hz_z *d_x,
  * and update, complex64 inner BiCGStab to 1e-5 with at most 1000 iterations,
  * at most 50 refinement steps, maxit capping the inner iterations in total,
  * the best iterate kept), each system at its own stage; the handles' complex64
- * copies are made on demand (synchronising).  Binary64 products run on each
- * handle's row blocks (the block-flat core of HZ_SPMV_FLAT64), complex64 and
+ * copies are made on demand (synchronising).  Binary64 systems that fit
+ * on chip together (HZ_SPMV_FLAT64P handles with one row per lane, no more
+ * systems than SMs) run side by side, each on SMs of its own; the workspace
+ * of such a sweep stays with its first handle.  Otherwise binary64 products
+ * run on each handle's row blocks (the block-flat core of HZ_SPMV_FLAT64), complex64 and
  * double-float ones with `group` lanes per row.  d_x[s] holds x0 on entry and
  * the solution on exit.  h_info has nsys entries.  Synchronises `stream`.
  * Errors: HZ_ERR_ARG (nsys outside 0..1024, unknown mode, null pointers),

@@ -103,6 +103,66 @@ __global__ void __launch_bounds__(kOpThreads) k_outer_flat(int nfblk, const int 
     }
 }
 
+// The same product on the row-per-lane layout: one warp per slice, lane = row,
+// so mu is loaded once per row and there is no row table; columns and x are
+// read coalesced, 8 steps in flight.  A slice's entries are contiguous in g:
+// up to kFlatCap of them are put in order in shared memory and written out in
+// full lines, a wider slice writes directly.  MEASURED_OUTER
+__global__ void __launch_bounds__(kOpThreads) k_outer_slices(int n, int nsl, const int *__restrict__ base,
+                                                             const int *__restrict__ diag,
+                                                             const int *__restrict__ scol,
+                                                             const int *__restrict__ rowptr,
+                                                             const unsigned *__restrict__ longs,
+                                                             const int *__restrict__ col,
+                                                             const double2 *__restrict__ mu,
+                                                             const double2 *__restrict__ x, double2 *__restrict__ g) {
+    __shared__ double2 sorted[kOpThreads / 32][kFlatCap];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int step = gridDim.x * (kOpThreads / 32);
+    for (int s = blockIdx.x * (kOpThreads / 32) + w; s < nsl; s += step) {
+        const int row = 32 * s + lane, b = __ldg(base + s), steps = __ldg(base + s + 1) - b;
+        const int k0 = __ldg(rowptr + 32 * s), cnt = __ldg(rowptr + min(n, 32 * s + 32)) - k0;
+        int beg = 0, d = -1;
+        double2 m = make_double2(0.0, 0.0);
+        if (row < n) {
+            beg = __ldg(rowptr + row) - k0;
+            d = __ldg(diag + row);
+            m = __ldg(mu + row);
+        }
+        const bool small = cnt <= kFlatCap;
+        double2 *out = small ? sorted[w] : g + k0;
+        for (int u0 = 0; u0 < steps; u0 += kOpGroup) {
+            int c[kOpGroup];
+            double2 xv[kOpGroup];
+#pragma unroll
+            for (int q = 0; q < kOpGroup; ++q)
+                c[q] = u0 + q < steps ? __ldg(scol + (size_t)32 * (b + u0 + q) + lane) : -1;
+#pragma unroll
+            for (int q = 0; q < kOpGroup; ++q) xv[q] = c[q] >= 0 ? __ldg(x + c[q]) : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int q = 0; q < kOpGroup; ++q) {
+                if (u0 + q >= steps) break;
+                const double2 v = neg_conj_mul(m, xv[q]);
+                // step u of a row: its entries in storage order without the
+                // diagonal one, which is in the last step
+                const int u = u0 + q, e = d < 0 ? u : u == steps - 1 ? d : u < d ? u : u + 1;
+                if (c[q] >= 0) out[beg + e] = v;
+            }
+        }
+        for (unsigned lm = longs ? __ldg(longs + s) : 0u; lm; lm &= lm - 1) {   // long rows: from the CSR arrays
+            const int l = __ffs(lm) - 1, e = __ldg(rowptr + 32 * s + l + 1);
+            const double2 ml = __ldg(mu + 32 * s + l);
+            for (int k = __ldg(rowptr + 32 * s + l) + lane; k < e; k += 32)
+                out[k - k0] = neg_conj_mul(ml, __ldg(x + __ldg(col + k)));
+        }
+        if (small) {
+            __syncwarp();
+            for (int i = lane; i < cnt; i += 32) g[k0 + i] = sorted[w][i];
+            __syncwarp();
+        }
+    }
+}
+
 // position of the diagonal entry of every row (-1 if absent)
 __global__ void k_find_diag(int n, const int *__restrict__ rowptr, const int *__restrict__ col, int *__restrict__ pos) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -154,6 +214,17 @@ extern "C" HZ_API hz_status hz_outer_on_pattern(const hz_mat *A, const hz_z *d_m
     HZ_CHECK(A, "hz_outer_on_pattern: null handle");
     if (A->n == 0 || A->nnz == 0) return HZ_OK;
     HZ_CHECK(d_mu && d_x && d_gradval, "hz_outer_on_pattern: null vector");
+    if (A->nsl) {
+        DevInfo d;
+        HZ_TRY(dev_info(&d));
+        const int grid = (int)std::max<int64_t>(
+            1, std::min<int64_t>((A->nsl + kOpThreads / 32 - 1) / (kOpThreads / 32), (int64_t)d.num_sms * 16));
+        k_outer_slices<<<grid, kOpThreads, 0, (cudaStream_t)stream>>>(A->n, A->nsl, A->sl_base, A->sl_diag, A->sl_col,
+                                                                      A->rowptr, A->sl_long, A->col, (const double2 *)d_mu,
+                                                                      (const double2 *)d_x, (double2 *)d_gradval);
+        HZ_CUDA(cudaGetLastError());
+        return HZ_OK;
+    }
     if (A->fblk) {   // every handle has its row blocks; the row-group kernel stays for the rest
         DevInfo d;
         HZ_TRY(dev_info(&d));

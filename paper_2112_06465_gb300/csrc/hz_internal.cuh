@@ -634,9 +634,11 @@ struct hz_mat {
     // [sl_base[s], sl_base[s+1]); entry u of a row sits in slot
     // 32 (sl_base[s] + u) + lane (column -1 past the row's end), the diagonal
     // entry in the slice's last step, the others in storage order; bit u of sl_mask[s] says
-    // that step u has a nonzero imaginary part
+    // that step u has a nonzero imaginary part.  The few rows far longer than
+    // the others leave their slots empty (sl_long).
     int32_t nsl = 0;               // slices (0: no such layout)
     int64_t sl_slots = 0;
+    void *sl_mem = nullptr;        // the arrays below but sl_val32
     int32_t *sl_base = nullptr;    // [nsl + 1]
     std::vector<int32_t> sl_base_h;   // the same on the host
     uint64_t *sl_mask = nullptr;   // [nsl]
@@ -645,6 +647,7 @@ struct hz_mat {
     double *sl_re = nullptr;       // [sl_slots]
     double *sl_im = nullptr;       // [sl_slots] (read where the mask says so)
     float2 *sl_val32 = nullptr;    // [sl_slots] complex64 copy, if c64
+    unsigned *sl_long = nullptr;   // [nsl] lanes of long rows, null without any
     // the handle has one of the two packed binary64 streams
     bool packed() const { return pk_re || sl_re; }
     int32_t nfblk_t = 0;       // the same for the bulk-copy kernel's smaller chunks

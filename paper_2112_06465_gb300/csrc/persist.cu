@@ -1092,6 +1092,7 @@ static cudaError_t ps_launch(PsKind kind, hz_mat *const *A, const PsSys *h, int 
 // binary32 pipes.  The CTAs (0: not this way) and their shared memory:
 static int ps_cluster(const hz_mat *A, PsKind kind, size_t *smem) {
     const PsMethod m = ps_method(kind);
+    if (A->sl_long) return 0;   // (their columns are not staged)
     int c = 1;
     while (c < kPsMaxCluster && c < A->nsl) c *= 2;
     const int per = (A->nsl + c - 1) / c;

@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(256) k_sl_fill(int n, int nsl, const int *__re
                                                  double2 *val, int first, int *__restrict__ diag,
                                                  int *__restrict__ scol, double *__restrict__ sre,
                                                  double *__restrict__ sim, unsigned long long *__restrict__ mask,
-                                                 float2 *__restrict__ v32, SetDiag sd) {
+                                                 float2 *__restrict__ v32, const unsigned *__restrict__ longs,
+                                                 SetDiag sd) {
     constexpr int G = 4;
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -145,14 +146,26 @@ __global__ void __launch_bounds__(256) k_sl_fill(int n, int nsl, const int *__re
         int beg = 0, len = 0, d = -1;
         if (row < n) {
             beg = rowptr[row];
-            len = min(w, max(0, rowptr[row + 1] - beg));
+            const int all = max(0, rowptr[row + 1] - beg);
             if (first) {
-                for (int k = 0; k < len && d < 0; ++k)
+                for (int k = 0; k < all && d < 0; ++k)
                     if (col[beg + k] == row) d = k;
                 diag[row] = d;
             } else {
                 d = diag[row];
             }
+            len = min(w, all);
+        }
+        double2 dv = make_double2(0.0, 0.0);
+        const bool newd = sd.theta && d >= 0;
+        if (newd) {
+            dv = sd.base[row];
+            cmac(dv, sd.c, sd.theta[row]);
+            val[beg + d] = dv;
+        }
+        if (longs && (longs[s] >> lane) & 1u) {   // a long row: no slots
+            len = 0;
+            d = -1;
         }
         unsigned long long m = 0ull;
         for (int u0 = 0; u0 < w; u0 += G) {
@@ -170,14 +183,9 @@ __global__ void __launch_bounds__(256) k_sl_fill(int n, int nsl, const int *__re
                 k[q] = e >= 0 ? beg + e : -1;
                 a[q] = k[q] >= 0 ? val[k[q]] : make_double2(0.0, 0.0);
             }
-            if (sd.theta && d >= 0 && u0 + G >= w) {
-                double2 v = sd.base[row];
-                cmac(v, sd.c, sd.theta[row]);
-                val[beg + d] = v;
 #pragma unroll
-                for (int q = 0; q < G; ++q)
-                    if (u0 + q == w - 1) a[q] = v;
-            }
+            for (int q = 0; q < G; ++q)
+                if (newd && d >= 0 && u0 + q == w - 1) a[q] = dv;
 #pragma unroll
             for (int q = 0; q < G; ++q) {
                 if (u0 + q >= w) break;
@@ -198,7 +206,7 @@ static hz_status sl_refresh(hz_mat *A, int first, const SetDiag &sd, cudaStream_
     HZ_TRY(dev_info(&d));
     k_sl_fill<<<stream_grid(d, (int64_t)A->nsl * 32, 256, 8), 256, 0, s>>>(
         A->n, A->nsl, A->sl_base, A->rowptr, A->col, A->val, first, A->sl_diag, A->sl_col, A->sl_re, A->sl_im,
-        (unsigned long long *)A->sl_mask, A->sl_val32, sd);
+        (unsigned long long *)A->sl_mask, A->sl_val32, A->sl_long, sd);
     HZ_CUDA(cudaGetLastError());
     return HZ_OK;
 }
@@ -270,7 +278,7 @@ MatView<double2> mat_view<double2>(const hz_mat *A) {
     v.pk_base = A->pk_base; v.pk_gbase = A->pk_gbase; v.pk_gim = A->pk_gim; v.pk_col = A->pk_col;
     v.pk_re = A->pk_re; v.pk_im = A->pk_im;
     v.nsl = A->nsl; v.sl_base = A->sl_base; v.sl_mask = (const unsigned long long *)A->sl_mask;
-    v.sl_col = A->sl_col; v.sl_re = A->sl_re; v.sl_im = A->sl_im;
+    v.sl_col = A->sl_col; v.sl_re = A->sl_re; v.sl_im = A->sl_im; v.sl_long = A->sl_long;
     return v;
 }
 
@@ -281,7 +289,7 @@ MatView<float2> mat_view<float2>(const hz_mat *A) {
     v.nfblk = A->nfblk; v.fblk = A->fblk; v.fblk_k = A->fblk_k;
     v.nchunks = A->sell_nchunks; v.chunk_off = A->sell_chunk_off; v.chunk_w = A->sell_chunk_w;
     v.perm = A->sell_perm; v.scol = A->sell_col; v.sval = A->sell_val32;
-    v.nsl = A->sl_val32 ? A->nsl : 0; v.sl_base = A->sl_base; v.sl_col = A->sl_col; v.sl_val32 = A->sl_val32;
+    v.nsl = A->sl_val32 ? A->nsl : 0; v.sl_base = A->sl_base; v.sl_col = A->sl_col; v.sl_val32 = A->sl_val32; v.sl_long = A->sl_long;
     return v;
 }
 
@@ -646,30 +654,54 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
     if (n > 0 && nnz > 0) {
         const int ns = (n + 31) / 32;
         std::vector<int> sb(ns + 1);
-        int64_t P = 0;
+        std::vector<unsigned> lg(ns, 0u);   // lanes of long rows
+        const double lim = std::max((double)kSlLongRow, 2.0 * A->mean_row);
+        int64_t P = 0, longs = 0, short_nnz = nnz;
         int wmax = 0;
         for (int q = 0; q < ns; ++q) {
             int w = 0;
-            for (int r = 32 * q; r < std::min(n, 32 * q + 32); ++r) w = std::max(w, rp[r + 1] - rp[r]);
+            for (int r = 32 * q; r < std::min(n, 32 * q + 32); ++r) {
+                const int len = rp[r + 1] - rp[r];
+                if (len > lim) {
+                    lg[q] |= 1u << (r & 31);
+                    longs += 1;
+                    short_nnz -= len;
+                } else {
+                    w = std::max(w, len);
+                }
+            }
             sb[q] = (int)std::min<int64_t>(P, INT32_MAX);
             P += w;
             wmax = std::max(wmax, w);
         }
         sb[ns] = (int)std::min<int64_t>(P, INT32_MAX);
         const int64_t slots = 32 * P;
-        if (wmax <= kSlMaxWidth && slots < INT32_MAX - 32 &&
-            (4 * slots <= 5 * (int64_t)nnz || (n <= 65536 && 5 * slots <= 7 * (int64_t)nnz))) {
+        // few long rows only: a warp sums its slice's one after the other
+        if (P > 0 && wmax <= kSlMaxWidth && mx <= kFlatCap && 128 * longs <= n && slots < INT32_MAX - 32 &&
+            (4 * slots <= 5 * short_nnz || (n <= 65536 && 5 * slots <= 7 * short_nnz))) {
             A->nsl = ns;
             A->sl_slots = slots;
             A->sl_base_h.assign(sb.begin(), sb.end());
-            if (cudaMalloc(&A->sl_base, sizeof(int) * (ns + 1)) != cudaSuccess ||
-                cudaMalloc(&A->sl_mask, sizeof(uint64_t) * ns) != cudaSuccess ||
-                cudaMalloc(&A->sl_diag, sizeof(int) * n) != cudaSuccess ||
-                cudaMalloc(&A->sl_col, sizeof(int) * slots) != cudaSuccess ||
-                cudaMalloc(&A->sl_re, sizeof(double) * slots) != cudaSuccess ||
-                cudaMalloc(&A->sl_im, sizeof(double) * slots) != cudaSuccess ||
-                ((flags & HZ_FLAG_C64) && cudaMalloc(&A->sl_val32, sizeof(float2) * slots) != cudaSuccess) ||
-                cudaMemcpy(A->sl_base, sb.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice) != cudaSuccess) {
+            // one allocation (creation is paid for by every new operator)
+            const size_t bytes[7] = {sizeof(double) * slots, sizeof(double) * slots, sizeof(uint64_t) * ns,
+                                     sizeof(int) * slots,    sizeof(int) * n,        sizeof(int) * (ns + 1),
+                                     longs ? sizeof(int) * ns : 0};
+            size_t at[8] = {0};
+            for (int q = 0; q < 7; ++q) at[q + 1] = (at[q] + bytes[q] + 255) & ~(size_t)255;
+            const bool ok = cudaMalloc(&A->sl_mem, at[7]) == cudaSuccess;
+            char *m = (char *)A->sl_mem;
+            if (ok) {
+                A->sl_re = (double *)(m + at[0]);
+                A->sl_im = (double *)(m + at[1]);
+                A->sl_mask = (uint64_t *)(m + at[2]);
+                A->sl_col = (int32_t *)(m + at[3]);
+                A->sl_diag = (int32_t *)(m + at[4]);
+                A->sl_base = (int32_t *)(m + at[5]);
+                if (longs) A->sl_long = (unsigned *)(m + at[6]);
+            }
+            if (!ok || ((flags & HZ_FLAG_C64) && cudaMalloc(&A->sl_val32, sizeof(float2) * slots) != cudaSuccess) ||
+                cudaMemcpy(A->sl_base, sb.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+                (longs && cudaMemcpy(A->sl_long, lg.data(), sizeof(int) * ns, cudaMemcpyHostToDevice) != cudaSuccess)) {
                 set_error("hz_csr_create: allocation failed");
                 return fail(HZ_ERR_ALLOC);
             }
@@ -807,12 +839,7 @@ extern "C" HZ_API hz_status hz_mat_destroy(hz_mat *A) {
     cudaFree(A->pk_col);
     cudaFree(A->pk_re);
     cudaFree(A->pk_im);
-    cudaFree(A->sl_base);
-    cudaFree(A->sl_mask);
-    cudaFree(A->sl_diag);
-    cudaFree(A->sl_col);
-    cudaFree(A->sl_re);
-    cudaFree(A->sl_im);
+    cudaFree(A->sl_mem);
     cudaFree(A->sl_val32);
     cudaFree(A->fblk_t);
     cudaFree(A->col_pad);

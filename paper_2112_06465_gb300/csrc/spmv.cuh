@@ -116,6 +116,7 @@ struct MatView {
     const double *sl_re;
     const double *sl_im;
     const float2 *sl_val32;
+    const unsigned *sl_long;   // lanes of each slice whose rows are long (null: none)
 };
 
 // Epilogue interface (every fused SpMV epilogue provides):
@@ -1050,6 +1051,12 @@ __device__ __forceinline__ void flat_rows_d64(const MatView<double2> &A, const d
 // operations a component and the NaN is set when the row ends.
 constexpr int kSlG = 8;            // steps whose loads are in flight together
 constexpr int kSlMaxWidth = 64;    // steps per slice at most (bits of the mask)
+// A row longer than this many entries and twice the mean leaves its slots
+// empty and is summed by all lanes of its slice's warp from the CSR arrays:
+// one such row in a slice would make every lane step through its length.
+// (618 k rows of 15, 161 of them 97 to 195 long: 115 us a product that way, 52
+// us this way, 60 us as lane runs.)
+constexpr int kSlLongRow = 32;
 // resident CTAs per SM asked of the register allocator
 template <class V> constexpr int kSlMinBlocks = std::is_same<V, double2>::value ? 4 : 8;
 
@@ -1166,6 +1173,9 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const Gather &gx
         for (int u = 0; u < G; ++u) c[u] = u0 + u < q.w ? ldm(p + 32 * u) : -1;
     };
     Sl cur = meta(s0), nxt = meta(s0 + step);
+    constexpr int kLongG = 4;
+    auto longs = [&](int s) { return A.sl_long && s < send ? __ldg(A.sl_long + s) : 0u; };
+    unsigned lcur = kLive != 3 ? longs(s0) : 0u, lnxt = kLive != 3 ? longs(s0 + step) : 0u;
     int cn[G];
     cols(cur, 0, cn);
     if (!wait()) return;
@@ -1214,6 +1224,33 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const Gather &gx
         if constexpr (kD) {
             if ((int)bad_re < 0) y.x = __longlong_as_double(0x7ff8000000000000ll);
             if ((int)bad_im < 0) y.y = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        if constexpr (kLive != 3) {   // (a cluster takes no matrix with long rows)
+            for (unsigned lm = lcur; lm; lm &= lm - 1) {
+                const int l = __ffs(lm) - 1, end = __ldg(A.rowptr + 32 * s + l + 1);
+                V t = czero<V>();
+                for (int k0 = __ldg(A.rowptr + 32 * s + l) + lane; k0 < end; k0 += 32 * kLongG) {
+                    int c[kLongG];
+                    V a[kLongG], v[kLongG];
+#pragma unroll
+                    for (int u = 0; u < kLongG; ++u) {
+                        c[u] = k0 + 32 * u < end ? __ldg(A.col + k0 + 32 * u) : -1;
+                        a[u] = k0 + 32 * u < end ? __ldg(A.val + k0 + 32 * u) : czero<V>();
+                    }
+#pragma unroll
+                    for (int u = 0; u < kLongG; ++u) v[u] = c[u] >= 0 ? gx(c[u]) : czero<V>();
+#pragma unroll
+                    for (int u = 0; u < kLongG; ++u) cmac(t, a[u], v[u]);
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    t.x += __shfl_xor_sync(0xffffffffu, t.x, off);
+                    t.y += __shfl_xor_sync(0xffffffffu, t.y, off);
+                }
+                if (lane == l) y = t;
+            }
+            lcur = lnxt;
+            lnxt = longs(s + 2 * step);
         }
         if (in) epi_row(epi, row, y, acc, pf);
         cur = nxt;
