@@ -126,3 +126,38 @@ def test_sweep_against_single_solves(hz, sizes):
         elif k < 4:
             y, _ = hz.zsolve(M, b, tol=TOL, maxit=200)
             assert float(torch.linalg.vector_norm(x - y) / torch.linalg.vector_norm(y)) <= 3.5 * TOL
+
+
+@pytest.mark.parametrize("n", [3000, 20011, 200003])
+def test_threads_and_streams(hz, n):
+    """Solves from two host threads on streams of their own, each on its own
+    handle (one cluster each; every SM each, vectors from a little to nearly
+    all of their shared memory), give the answers of the same solves alone."""
+    import threading
+
+    mats = [hz.Matrix.from_csr(operator(n, 90 + k)) for k in range(2)]
+    bs = [vec(n, 95 + k) for k in range(2)]
+    alone = [hz.zsolve(M, b, tol=TOL, maxit=200)[0] for M, b in zip(mats, bs)]
+    torch.cuda.synchronize()
+    out, errors = [[], []], []
+
+    def work(k):
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                for _ in range(20):
+                    x, info = hz.zsolve(mats[k], bs[k], tol=TOL, maxit=200)
+                    assert info.status == 0
+                    out[k].append(x)
+            s.synchronize()
+        except Exception as e:   # reported below, in the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for k in range(2):
+        assert len(out[k]) == 20 and all(torch.equal(x, alone[k]) for x in out[k])
