@@ -835,7 +835,7 @@ extern "C" HZ_API hz_status hz_zsolve_batched(int32_t nsys, hz_mat *const *A, co
         if (mixed && A[k]->n > 0) HZ_TRY(ensure_c64(A[k], s));
     }
     // binary64 systems whose vectors fit on chip: each on CTAs of its own
-    // (12 boxes of 12^3 to 24^3: 3.5 ms, in the phases below 10.4 ms); more
+    // (12 boxes of 15^3 to 24^3: 3.7 ms, in the phases below 10.4 ms); more
     // systems than SMs, larger ones and the other formats take the phases
     std::vector<int> ncta;
     if (!mixed && !ff && ps_batch_plan(A, nsys, &ncta)) {

@@ -34,9 +34,9 @@
 // shuffle sums and the scalars on one thread: 12 000 cycles per barrier, 35
 // us per BiCGStab iteration on 4096 unknowns.)
 //
-// Measured against the graphs, whole solves: BiCGStab on 16^3 unknowns 3.2 ->
-// 1.66 ms, on 64^3 25.0 -> 16.5 ms; mixed on 48^3 13.0 -> 5.3 ms; forward and
-// adjoint TFQMR on 32^3 26.5 -> 14.4 ms.
+// Measured against the graphs, whole solves: BiCGStab on 16^3 unknowns 3.1 ->
+// 1.66 ms (1.31 ms on one cluster, below), on 64^3 25.4 -> 15.9 ms; mixed on
+// 48^3 12.5 -> 5.3 ms; forward and adjoint TFQMR on 32^3 26.7 -> 14.5 ms.
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -1229,7 +1229,7 @@ hz_status ps_solve(hz_mat *A, PsKind kind, const Ctl &c, Info *out, int *restart
 // only, instead of advancing together through grid-wide phases
 // (batched.cu, 75 to 95 us per iteration for any sweep of small systems).
 // CTAs are shared out by rows, one more at a time to the system whose CTAs
-// own the most slices.  Twelve boxes of 12^3 to 24^3 unknowns: 10.4 -> 3.5 ms.
+// own the most slices.  Twelve boxes of 15^3 to 24^3 unknowns: 10.4 -> 3.7 ms.
 struct PsBatch {
     std::atomic_flag busy = ATOMIC_FLAG_INIT;
     void *mem = nullptr;
