@@ -334,9 +334,12 @@ struct PsState {
     double nb;
     double rel;        // the residual ratio, or, with lazy set,
     double rr;         // the squared residual norm it follows from
-    double thr;        // squared norms above it have not converged
+    double thr, top;   // squared norms in (thr, top] have not converged and have a finite ratio
     int iter, done, half, status, zero_x, lazy;
     __device__ double ratio() const { return lazy ? sqrt(rr) / nb : rel; }
+    // whether a squared norm needs no exact test.  (Every CTA decides the same:
+    // nothing that only one of them has, the history for one, enters.)
+    __device__ bool clear(double ss) const { return ss > thr && ss <= top; }
 };
 
 // the threshold for squared norms of the test rel <= tol: a little above
@@ -344,6 +347,11 @@ struct PsState {
 __device__ __forceinline__ double ps_threshold(double tol, double nb) {
     const double t = tol * nb, t2 = t * t * 1.000001;
     return t2 > 1e-290 ? t2 : 1e-290;
+}
+// squared norms up to it over nb^2 are at most 1e600: the ratio does not overflow
+__device__ __forceinline__ double ps_top(double nb) {
+    const double t = 1e300 * nb;
+    return fmin(t * t, 1.7976931348623157e308);
 }
 
 // the BiCGStab iterations from r, rh, p = v = 0 in shared memory until the
@@ -411,12 +419,7 @@ __device__ bool ps_bicg_loop(const MatView<V> &A, const Ctl &ctl, const Own &o, 
             [&]() {
                 return grp_reduce<kLive, R, 1, true>(g, sh, ssum, [&](R(&tot)[1], int lane) {
                            const double ss = (double)tot[0];
-                           if (lane != 0 || ss > st.thr) {
-                               if (lane == 0 && !finite_d(ss)) {
-                                   st.status = HZ_ERR_NAN; st.done = 1; st.rel = ss; st.lazy = 0;
-                               }
-                               return;
-                           }
+                           if (lane != 0 || st.clear(ss)) return;
                            const double rel = sqrt(ss) / st.nb;
                            if (!finite_d(rel)) { st.status = HZ_ERR_NAN; st.done = 1; st.rel = rel; st.lazy = 0; }
                            else if (kOuter ? rel <= ctl.tol : (float)rel <= ctl.inner_tol) {
@@ -483,9 +486,11 @@ __device__ bool ps_bicg_loop(const MatView<V> &A, const Ctl &ctl, const Own &o, 
                     const bool last = it >= maxit || (!kOuter && *total >= ctl.maxit);
                     st.rr = rr;
                     st.lazy = 1;
-                    if (rr > st.thr && finite_d(rr) && !last && !hist && !cis_zero(omega)) return;
+                    const bool go = st.clear(rr) && !last && !cis_zero(omega);
+                    if (go && !hist) return;
                     const double rel = sqrt(rr) / st.nb;
                     if (hist) ctl.hist[it] = rel;
+                    if (go) return;
                     if (!finite_d(rel)) { st.status = HZ_ERR_NAN; st.done = 1; }
                     else if (kOuter ? rel <= ctl.tol : (float)rel <= ctl.inner_tol) { st.status = HZ_OK; st.done = 1; }
                     else if (cis_zero(omega)) { st.status = HZ_BREAKDOWN; st.done = 1; }
@@ -516,6 +521,7 @@ __device__ __forceinline__ void ps_start_state(const Ctl &ctl, PsState<double2> 
     const double2 one = make_double2(1.0, 0.0);
     st.nb = nb;
     st.thr = ps_threshold(ctl.tol, nb);
+    st.top = ps_top(nb);
     st.half = 0;
     st.lazy = 0;
     st.rho = make_double2(rr, 0.0);
@@ -759,6 +765,7 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_mixed(const PsSys *s
                     in.beta = make_float2(0.f, 0.f);
                     in.nb = (double)sqrtf((float)tot[2]);
                     in.thr = ps_threshold((double)ctl.inner_tol, in.nb);
+                    in.top = ps_top(in.nb);
                     in.rel = 1.0; in.lazy = 0;
                     in.iter = 0; in.half = 0; in.status = HZ_NOT_CONVERGED;
                     in.done = in.nb == 0.0 ? 1 : 0;
@@ -984,9 +991,11 @@ __global__ void __launch_bounds__(kPsMaxWarps * 32, 1) k_ps_tfqmr(const PsSys *s
                 const double rr = ((double)q.m + 1.0) * (q.tau2 * q.xs) * q.xs;
                 st.rr = rr;
                 st.lazy = 1;
-                if (rr > st.thr && finite_d(rr) && !hist) return;
+                const bool go = st.clear(rr);
+                if (go && !hist) return;
                 const double rel = sqrt(rr) / st.nb;
                 if (hist) ctl.hist[it] = rel;
+                if (go) return;
                 if (!finite_d(rel)) { st.status = HZ_ERR_NAN; q.stop = 1; }
                 else if (rel <= ctl.tol) { st.status = HZ_OK; q.stop = 1; }
             }))

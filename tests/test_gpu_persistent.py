@@ -161,3 +161,34 @@ def test_threads_and_streams(hz, n):
     assert not errors, errors
     for k in range(2):
         assert len(out[k]) == 20 and all(torch.equal(x, alone[k]) for x in out[k])
+
+
+@pytest.mark.parametrize("n", [1000, 20011])   # one cluster; every SM
+@pytest.mark.parametrize("method", ["bicgstab", "tfqmr"])
+def test_overflowing_ratio(hz, n, method):
+    """A residual ratio that overflows while its square is finite ends the
+    solve on every CTA alike, with a history (which one CTA writes) or without.
+
+    ||b|| = 2^-530 and a start with ||r0|| = 1.5e308 ||b||; A = S + 0.01 I with
+    S real and skew, so that alpha = 100 for a real r0 and the first step makes
+    the residual larger (TFQMR's bound grows with sqrt(m + 1))."""
+    i = np.arange(n - 1, dtype=np.int32)
+    rows = np.concatenate([i, np.arange(n), i + 1])
+    cols = np.concatenate([i + 1, np.arange(n), i])
+    vals = np.concatenate([np.ones(n - 1), np.full(n, 0.01), -np.ones(n - 1)]) + 0j
+    order = np.lexsort((cols, rows))
+    rp = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=n))]).astype(np.int32)
+    A = W.CSR(n, rp, cols[order].astype(np.int32), vals[order])
+    x0 = np.random.default_rng(n).standard_normal(n) + 0j
+    b = np.zeros(n, np.complex128)
+    b[0] = 2.0 ** -530
+    x0 *= 1.5e308 * 2.0 ** -530 / np.linalg.norm(A.to_scipy() @ x0)
+    M = hz.Matrix.from_csr(A)
+    for hist in (None, torch.zeros(51, dtype=torch.float64, device="cuda")):
+        _, info = hz.zsolve(M, torch.as_tensor(b).cuda(), x=torch.as_tensor(x0).cuda(), tol=1e-10, maxit=50,
+                            method=method, hist=hist)
+        assert info.status == 6 and info.iters == 1, info
+    assert np.isfinite(float(hist[0]))
+    if method == "tfqmr":   # (BiCGStab ends in the half step, which writes none)
+        assert not np.isfinite(float(hist[1]))
+    M.close()
