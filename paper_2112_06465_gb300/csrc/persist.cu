@@ -1309,12 +1309,13 @@ hz_status ps_solve_batched(hz_mat *const *A, int ns, const std::vector<int> &nct
     const size_t bytes = zero_b + sys_b + vec_b;
     // the workspace stays with the first handle; a call that finds it in use
     // (another thread sweeping over the same handles) takes its own
-    if (!act[0]->ps_batch) {
-        static std::mutex mu;
+    PsBatch *B;
+    {
+        static std::mutex mu;   // (the pointer is read under it too: another thread may be setting it)
         std::lock_guard<std::mutex> lk(mu);
         if (!act[0]->ps_batch) act[0]->ps_batch = new PsBatch();
+        B = (PsBatch *)act[0]->ps_batch;
     }
-    PsBatch *B = (PsBatch *)act[0]->ps_batch;
     const bool mine = !B->busy.test_and_set(std::memory_order_acquire);
     char *mem = nullptr;
     cudaError_t e = cudaSuccess;

@@ -192,3 +192,38 @@ def test_overflowing_ratio(hz, n, method):
     if method == "tfqmr":   # (BiCGStab ends in the half step, which writes none)
         assert not np.isfinite(float(hist[1]))
     M.close()
+
+
+def test_threads_sweep_the_same_handles(hz):
+    """Two host threads, on streams of their own, sweep over the same handles
+    from their first sweep on (the workspace kept with the first handle serves
+    one of them at a time): the answers are those of the sweep alone."""
+    import threading
+
+    mats = [hz.Matrix.from_csr(operator(n, 60 + n)) for n in (4865, 700, 9001)]
+    bs = [vec(M.n, 70 + k) for k, M in enumerate(mats)]
+    torch.cuda.synchronize()
+    out, errors, gate = [[], []], [], threading.Barrier(2)
+
+    def work(k):
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                gate.wait()
+                for _ in range(20):
+                    xs, infos = hz.zsolve_batched(mats, bs, tol=TOL, maxit=200)
+                    assert all(i.status == 0 for i in infos)
+                    out[k].append(xs)
+            s.synchronize()
+        except Exception as e:   # reported below, in the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    alone, _ = hz.zsolve_batched(mats, bs, tol=TOL, maxit=200)
+    for o in out:
+        assert len(o) == 20 and all(torch.equal(x, y) for xs in o for x, y in zip(xs, alone))
