@@ -1,0 +1,83 @@
+// plan.h -- decisions of the host side that need no device: which matrices get
+// the row-per-lane layout.  Plain C++, so that a test compiles it by itself.
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+#include <vector>
+
+namespace hz {
+
+constexpr int kSlMaxWidth = 64;    // steps per slice at most (bits of the mask)
+constexpr int kSlMaxRow = 512;     // entries of a long row at most
+// A row longer than this many entries and twice the mean leaves its slots
+// empty and is summed by all lanes of its slice's warp from the CSR arrays:
+// one such row in a slice would make every lane step through its length.
+// (618 k rows of 15, 161 of them 97 to 195 long: 115 us a product that way, 52
+// us this way, 60 us as lane runs.)
+constexpr int kSlLongRow = 32;
+constexpr int kSlLongG = 8;        // loads of such a row in flight per lane: 256 entries a pass
+// The warp takes its long rows one after the other, so long rows that lie
+// together keep one warp busy while the others have finished: at most this
+// many passes over all long rows of a slice.  us a product from cold caches,
+// 20 k rows of 15 with some of 400 side by side (lane runs 15.0, without long
+// rows 10.9), four loads in flight: 1 row 17, 2 rows 23, 8 rows 62, 32 rows
+// 165, and a BiCGStab iteration with 32 of them 261 against the graph's 53;
+// eight in flight: 1 row 15, 2 rows of 255 17.
+constexpr int kSlLongPasses = 2;
+
+// The row-per-lane layout of a CSR pattern: slices of 32 rows, one per lane,
+// as wide as the slice's longest row that is not a long one.
+struct SlicePlan {
+    bool fits = false;
+    std::vector<int32_t> base;     // [slices + 1] first step of each slice
+    std::vector<unsigned> longs;   // [slices] lanes of long rows
+    int64_t slots = 0;
+    int64_t nlong = 0;
+};
+
+// Padded rows cost binary64 instructions, so the padded size may exceed the
+// entries by a quarter (the lane-run stream's row switches and second
+// accumulator cost it 26 % more binary64 instructions than the multiply-adds
+// it needs: 728 k against 577 k on 618 k rows of 15), by two fifths where the
+// work is small and launches and latency count instead: rows of 9 to 17 in
+// random order, padded by 1.3, lane runs / slices, a product 9.0 / 5.6 us at
+// 4,000 rows and 15.1 / 8.2 at 64,000, a BiCGStab iteration 54 / 25 and 78 /
+// 42.
+inline SlicePlan slice_plan(const int32_t *rp, int32_t n, int32_t nnz) {
+    SlicePlan p;
+    if (n <= 0 || nnz <= 0) return p;
+    const int ns = (n + 31) / 32;
+    p.base.resize(ns + 1);
+    p.longs.assign(ns, 0u);
+    const double lim = std::max((double)kSlLongRow, 2.0 * ((double)nnz / n));
+    int64_t P = 0, short_nnz = nnz;
+    int wmax = 0, rmax = 0, passes_max = 0;
+    for (int q = 0; q < ns; ++q) {
+        int w = 0, passes = 0;
+        for (int r = 32 * q; r < std::min(n, 32 * q + 32); ++r) {
+            const int len = rp[r + 1] - rp[r];
+            rmax = std::max(rmax, len);
+            if (len > lim) {
+                p.longs[q] |= 1u << (r & 31);
+                p.nlong += 1;
+                short_nnz -= len;
+                passes += (len + 32 * kSlLongG - 1) / (32 * kSlLongG);
+            } else {
+                w = std::max(w, len);
+            }
+        }
+        p.base[q] = (int32_t)std::min<int64_t>(P, INT32_MAX);
+        P += w;
+        wmax = std::max(wmax, w);
+        passes_max = std::max(passes_max, passes);
+    }
+    p.base[ns] = (int32_t)std::min<int64_t>(P, INT32_MAX);
+    p.slots = 32 * P;
+    p.fits = P > 0 && wmax <= kSlMaxWidth && rmax <= kSlMaxRow && 128 * p.nlong <= n && passes_max <= kSlLongPasses &&
+             p.slots < INT32_MAX - 32 &&
+             (4 * p.slots <= 5 * short_nnz || (n <= 65536 && 5 * p.slots <= 7 * short_nnz));
+    return p;
+}
+
+}  // namespace hz

@@ -645,43 +645,16 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
         set_error("hz_csr_create: allocation failed");
         return fail(HZ_ERR_ALLOC);
     }
-    // the row-per-lane stream where it fits: padded rows cost binary64
-    // instructions, so the padded size may exceed the entries by a quarter
-    // (the lane-run stream's row switches and second accumulator cost it 26 %
-    // more binary64 instructions than the multiply-adds it needs: 728 k
-    // against 577 k on 618 k rows of 15), by two fifths where the work is
-    // small and launches and latency count instead
-    if (n > 0 && nnz > 0) {
-        const int ns = (n + 31) / 32;
-        std::vector<int> sb(ns + 1);
-        std::vector<unsigned> lg(ns, 0u);   // lanes of long rows
-        const double lim = std::max((double)kSlLongRow, 2.0 * A->mean_row);
-        int64_t P = 0, longs = 0, short_nnz = nnz;
-        int wmax = 0;
-        for (int q = 0; q < ns; ++q) {
-            int w = 0;
-            for (int r = 32 * q; r < std::min(n, 32 * q + 32); ++r) {
-                const int len = rp[r + 1] - rp[r];
-                if (len > lim) {
-                    lg[q] |= 1u << (r & 31);
-                    longs += 1;
-                    short_nnz -= len;
-                } else {
-                    w = std::max(w, len);
-                }
-            }
-            sb[q] = (int)std::min<int64_t>(P, INT32_MAX);
-            P += w;
-            wmax = std::max(wmax, w);
-        }
-        sb[ns] = (int)std::min<int64_t>(P, INT32_MAX);
-        const int64_t slots = 32 * P;
-        // few long rows only: a warp sums its slice's one after the other
-        if (P > 0 && wmax <= kSlMaxWidth && mx <= kFlatCap && 128 * longs <= n && slots < INT32_MAX - 32 &&
-            (4 * slots <= 5 * short_nnz || (n <= 65536 && 5 * slots <= 7 * short_nnz))) {
+    // the row-per-lane stream where it fits
+    {
+        const SlicePlan sp = slice_plan(rp.data(), n, nnz);
+        if (sp.fits) {
+            const int ns = (int)sp.longs.size();
+            const int64_t slots = sp.slots;
+            const bool longs = sp.nlong > 0;
             A->nsl = ns;
             A->sl_slots = slots;
-            A->sl_base_h.assign(sb.begin(), sb.end());
+            A->sl_base_h = sp.base;
             // one allocation (creation is paid for by every new operator)
             const size_t bytes[7] = {sizeof(double) * slots, sizeof(double) * slots, sizeof(uint64_t) * ns,
                                      sizeof(int) * slots,    sizeof(int) * n,        sizeof(int) * (ns + 1),
@@ -700,8 +673,9 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
                 if (longs) A->sl_long = (unsigned *)(m + at[6]);
             }
             if (!ok || ((flags & HZ_FLAG_C64) && cudaMalloc(&A->sl_val32, sizeof(float2) * slots) != cudaSuccess) ||
-                cudaMemcpy(A->sl_base, sb.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
-                (longs && cudaMemcpy(A->sl_long, lg.data(), sizeof(int) * ns, cudaMemcpyHostToDevice) != cudaSuccess)) {
+                cudaMemcpy(A->sl_base, sp.base.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+                (longs &&
+                 cudaMemcpy(A->sl_long, sp.longs.data(), sizeof(int) * ns, cudaMemcpyHostToDevice) != cudaSuccess)) {
                 set_error("hz_csr_create: allocation failed");
                 return fail(HZ_ERR_ALLOC);
             }

@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "arith.cuh"
+#include "plan.h"
 
 namespace hz {
 
@@ -56,6 +57,7 @@ constexpr int kFlatThreads = HZ_FLAT_THREADS;   // warps per CTA = kFlatThreads 
 constexpr int kFlatU = HZ_FLAT_U;
 constexpr int kFlatGroup = HZ_FLAT_GROUP;       // entries per lane whose loads are in flight together
 constexpr int kFlatCap = 32 * kFlatU;           // entries per warp row block
+static_assert(kFlatCap == kSlMaxRow, "the longest row of both packed layouts");
 constexpr int kFlatRows = 32;                   // rows per row block (one per lane in phase 2)
 static_assert(kFlatU % kFlatGroup == 0, "kFlatU must be a multiple of kFlatGroup");
 #ifndef HZ_FLAT_CONTIG
@@ -1050,13 +1052,6 @@ __device__ __forceinline__ void flat_rows_d64(const MatView<double2> &A, const d
 // it would be NaN, so the exponent fields of x are watched with two integer
 // operations a component and the NaN is set when the row ends.
 constexpr int kSlG = 8;            // steps whose loads are in flight together
-constexpr int kSlMaxWidth = 64;    // steps per slice at most (bits of the mask)
-// A row longer than this many entries and twice the mean leaves its slots
-// empty and is summed by all lanes of its slice's warp from the CSR arrays:
-// one such row in a slice would make every lane step through its length.
-// (618 k rows of 15, 161 of them 97 to 195 long: 115 us a product that way, 52
-// us this way, 60 us as lane runs.)
-constexpr int kSlLongRow = 32;
 // resident CTAs per SM asked of the register allocator
 template <class V> constexpr int kSlMinBlocks = std::is_same<V, double2>::value ? 4 : 8;
 
@@ -1173,7 +1168,6 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const Gather &gx
         for (int u = 0; u < G; ++u) c[u] = u0 + u < q.w ? ldm(p + 32 * u) : -1;
     };
     Sl cur = meta(s0), nxt = meta(s0 + step);
-    constexpr int kLongG = 4;
     auto longs = [&](int s) { return A.sl_long && s < send ? __ldg(A.sl_long + s) : 0u; };
     unsigned lcur = kLive != 3 ? longs(s0) : 0u, lnxt = kLive != 3 ? longs(s0 + step) : 0u;
     int cn[G];
@@ -1229,18 +1223,18 @@ __device__ __forceinline__ void slice_rows(const MatView<V> &A, const Gather &gx
             for (unsigned lm = lcur; lm; lm &= lm - 1) {
                 const int l = __ffs(lm) - 1, end = __ldg(A.rowptr + 32 * s + l + 1);
                 V t = czero<V>();
-                for (int k0 = __ldg(A.rowptr + 32 * s + l) + lane; k0 < end; k0 += 32 * kLongG) {
-                    int c[kLongG];
-                    V a[kLongG], v[kLongG];
+                for (int k0 = __ldg(A.rowptr + 32 * s + l) + lane; k0 < end; k0 += 32 * kSlLongG) {
+                    int c[kSlLongG];
+                    V a[kSlLongG], v[kSlLongG];
 #pragma unroll
-                    for (int u = 0; u < kLongG; ++u) {
+                    for (int u = 0; u < kSlLongG; ++u) {
                         c[u] = k0 + 32 * u < end ? __ldg(A.col + k0 + 32 * u) : -1;
                         a[u] = k0 + 32 * u < end ? __ldg(A.val + k0 + 32 * u) : czero<V>();
                     }
 #pragma unroll
-                    for (int u = 0; u < kLongG; ++u) v[u] = c[u] >= 0 ? gx(c[u]) : czero<V>();
+                    for (int u = 0; u < kSlLongG; ++u) v[u] = c[u] >= 0 ? gx(c[u]) : czero<V>();
 #pragma unroll
-                    for (int u = 0; u < kLongG; ++u) cmac(t, a[u], v[u]);
+                    for (int u = 0; u < kSlLongG; ++u) cmac(t, a[u], v[u]);
                 }
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) {

@@ -160,3 +160,50 @@ def test_nonfinite_x(hz, oracle):
     ok = np.isfinite(ref.real) & np.isfinite(ref.imag)
     assert np.allclose(y[ok], ref[ok], rtol=0, atol=1e-12)
     M.close()
+
+
+def on_slices(hz, A, x):
+    """Whether a product of the default kind reads the row-per-lane layout: lane
+    runs form the same sums as the unpacked kind, one row per lane other ones."""
+    M = hz.Matrix.from_csr(A)
+    y = host(hz.zspmv(M, dev(x)))
+    M.set_spmv("flat64")
+    same = np.array_equal(y, host(hz.zspmv(M, dev(x))))
+    M.close()
+    return not same
+
+
+def with_long(A, first, count, length, seed):
+    """A with `count` neighbouring rows replaced by rows of `length` entries."""
+    rng = np.random.default_rng(seed)
+    rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
+    keep = (rows < first) | (rows >= first + count)
+    r, c, v = [rows[keep]], [A.col[keep]], [A.val[keep]]
+    for i in range(first, first + count):
+        q = rng.permutation(A.n)
+        q = np.append(q[q != i][:length - 1], i)
+        r.append(np.full(length, i))
+        c.append(q)
+        v.append(rng.standard_normal(length) + 0j)
+    r, c, v = (np.concatenate(q) for q in (r, c, v))
+    o = np.lexsort((c, r))
+    rp = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=A.n))]).astype(np.int32)
+    return W.CSR(A.n, rp, c[o].astype(np.int32), v[o])
+
+
+@pytest.mark.parametrize("count,length,slices", [
+    (1, 255, True), (1, 257, True), (1, 512, True), (2, 256, True), (2, 257, False), (3, 100, False),
+    (32, 400, False)])
+def test_long_rows_together(hz, oracle, count, length, slices):
+    """Rows of up to two passes of 256 entries in a slice are summed by its
+    warp; more of them, which one warp would walk through alone, take the lane
+    runs."""
+    A = with_long(banded(5000, 9, 3, real=False), 1024, count, length, 17)
+    x = K.vectors(A.n, 18)[0]
+    assert on_slices(hz, A, x) == slices
+    M = hz.Matrix.from_csr(A, c64=True)
+    assert np.all(np.abs(host(hz.zspmv(M, dev(x))) - oracle.zspmv(A, x)) <= bound(A, x))
+    x32 = x.astype(np.complex64)
+    err = np.abs(host(hz.cspmv(M, dev(x32))) - oracle.cspmv(A, x32))
+    assert np.all(err <= bound(A, x32.astype(np.complex128), 2.0 ** -23))
+    M.close()

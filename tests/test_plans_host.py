@@ -1,0 +1,88 @@
+"""Host decisions of csrc/plan.h, compiled by themselves: the row-per-lane
+layout."""
+
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SOURCE = r"""
+#include "plan.h"
+using namespace hz;
+extern "C" int slices(const int *rp, int n, int *base, unsigned *longs, long long *slots) {
+    const SlicePlan p = slice_plan(rp, n, rp[n]);
+    std::copy(p.base.begin(), p.base.end(), base);
+    std::copy(p.longs.begin(), p.longs.end(), longs);
+    *slots = p.slots;
+    return p.fits;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    src, lib = str(d / "plan.cpp"), str(d / "plan.so")
+    with open(src, "w") as f:
+        f.write(SOURCE)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", "-I",
+                    os.path.join(ROOT, "paper_2112_06465_gb300", "csrc"), src, "-o", lib], check=True)
+    return C.CDLL(lib)
+
+
+def pointers(lens):
+    return np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+
+
+def slices(plan, lens):
+    rp, n = pointers(lens), len(lens)
+    ns = (n + 31) // 32
+    base, longs, slots = np.zeros(ns + 1, np.int32), np.zeros(ns, np.uint32), C.c_longlong()
+    fits = plan.slices(rp.ctypes.data_as(C.c_void_p), n, base.ctypes.data_as(C.c_void_p),
+                       longs.ctypes.data_as(C.c_void_p), C.byref(slots))
+    return bool(fits), base, longs, slots.value
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 95, 4099])
+@pytest.mark.parametrize("lo,hi,far", [(7, 7, 0), (0, 9, 0), (9, 17, 0), (5, 9, 100), (64, 64, 0), (65, 65, 0)])
+def test_slice_widths_and_long_rows(plan, n, lo, hi, far):
+    """Widths, long rows and slots against their definition, row by row."""
+    rng = np.random.default_rng(n + hi)
+    lens = rng.integers(lo, hi + 1, n)
+    if far:
+        lens[rng.integers(0, n, 1 + n // 100)] = far
+    if lens.sum() == 0:
+        lens[0] = 1
+    fits, base, longs, slots = slices(plan, lens)
+    lim = max(32.0, 2.0 * lens.sum() / n)
+    pad = np.zeros((len(longs), 32), int)
+    pad.reshape(-1)[:n] = lens
+    isl = pad > lim
+    assert np.array_equal((isl * (1 << np.arange(32, dtype=np.uint64))).sum(1), longs)
+    width = np.where(isl, 0, pad).max(1)
+    assert np.array_equal(np.concatenate([[0], np.cumsum(width)]), base) and slots == 32 * width.sum()
+    if width.max() > 64 or slots * 5 > 7 * (lens.sum() - pad[isl].sum()):
+        assert not fits
+
+
+@pytest.mark.parametrize("count,length,fits", [
+    (1, 33, True), (1, 512, True), (1, 513, False), (2, 256, True), (2, 257, False), (1, 257, True),
+    (3, 33, False), (8, 400, False), (32, 100, False)])
+def test_long_rows_that_lie_together(plan, count, length, fits):
+    """A warp sums its slice's long rows one after the other: at most two
+    passes of 256 entries over them, wherever the slice lies."""
+    for n in (8000, 600000):
+        for first in (0, 64, n - count):
+            lens = np.full(n, 7)
+            lens[first:first + count] = length
+            assert slices(plan, lens)[0] == fits
+        lens = np.full(n, 7)
+        lens[:128 * count:128] = 100   # one in a slice, any number of slices
+        assert slices(plan, lens)[0]
+    lens = np.full(8000, 7)
+    lens[:64 * 63:64] = 100            # more than one row in 128
+    assert not slices(plan, lens)[0]
