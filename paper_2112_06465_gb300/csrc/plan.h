@@ -54,17 +54,26 @@ inline SlicePlan slice_plan(const int32_t *rp, int32_t n, int32_t nnz) {
     int64_t P = 0, short_nnz = nnz;
     int wmax = 0, rmax = 0, passes_max = 0;
     for (int q = 0; q < ns; ++q) {
+        const int r0 = 32 * q, r1 = std::min(n, r0 + 32);
         int w = 0, passes = 0;
-        for (int r = 32 * q; r < std::min(n, 32 * q + 32); ++r) {
-            const int len = rp[r + 1] - rp[r];
-            rmax = std::max(rmax, len);
-            if (len > lim) {
-                p.longs[q] |= 1u << (r & 31);
-                p.nlong += 1;
-                short_nnz -= len;
-                passes += (len + 32 * kSlLongG - 1) / (32 * kSlLongG);
-            } else {
-                w = std::max(w, len);
+        const int32_t *row = rp + r0;
+        if (r1 - r0 == 32)   // (a loop that vectorises: every row of every new operator passes here)
+            for (int r = 0; r < 32; ++r) w = std::max(w, row[r + 1] - row[r]);
+        else
+            for (int r = 0; r < r1 - r0; ++r) w = std::max(w, row[r + 1] - row[r]);
+        rmax = std::max(rmax, w);
+        if (w > lim) {
+            w = 0;
+            for (int r = r0; r < r1; ++r) {
+                const int len = rp[r + 1] - rp[r];
+                if (len > lim) {
+                    p.longs[q] |= 1u << (r & 31);
+                    p.nlong += 1;
+                    short_nnz -= len;
+                    passes += (len + 32 * kSlLongG - 1) / (32 * kSlLongG);
+                } else {
+                    w = std::max(w, len);
+                }
             }
         }
         p.base[q] = (int32_t)std::min<int64_t>(P, INT32_MAX);
