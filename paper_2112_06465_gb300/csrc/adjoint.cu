@@ -103,23 +103,26 @@ __global__ void __launch_bounds__(kOpThreads) k_outer_flat(int nfblk, const int 
     }
 }
 
-// The same product on the row-per-lane layout: one warp per slice, lane = row,
-// so mu is loaded once per row and there is no row table; columns and x are
-// read coalesced, 8 steps in flight.  A slice's entries are contiguous in g:
-// up to kFlatCap of them are put in order in shared memory and written out in
-// full lines, a wider slice writes directly.
-// 64^3 box: 18.4 us, 20.5 us on the row blocks (from warm caches; the binary64
-// pipe's time is 13.8).
+// The same product on the row-per-lane layout, for slices of at most
+// kOpSliceCap entries: one warp per slice, lane = row, so mu is loaded once per
+// row and there is no row table; columns and x are read coalesced, 8 steps in
+// flight.  A slice's entries are contiguous in g: they are put in order in
+// shared memory and written out in full lines.  us warm, row blocks / slices:
+// 64^3 box 18.4 / 15.9 (binary64 pipe 13.8), 80^3 35.2 / 29.5, the same with
+// its rows and columns in random order 34.7 / 30.1.  Wider slices stay with the
+// row blocks: with staging for 512 entries too few warps are left to hide the
+// gathers (618 k rows of 15 in random order 81 -> 113 us), and slices written
+// directly scatter (672 k rows of 27: 146 -> 214 us).
+constexpr int kOpSliceCap = 256;
 __global__ void __launch_bounds__(kOpThreads) k_outer_slices(int n, int nsl, const int *__restrict__ base,
                                                              const int *__restrict__ diag,
                                                              const int *__restrict__ scol,
                                                              const int *__restrict__ rowptr,
-                                                             const unsigned *__restrict__ longs,
-                                                             const int *__restrict__ col,
                                                              const double2 *__restrict__ mu,
                                                              const double2 *__restrict__ x, double2 *__restrict__ g) {
-    __shared__ double2 sorted[kOpThreads / 32][kFlatCap];
+    __shared__ double2 sorted[kOpThreads / 32][kOpSliceCap];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double2 *out = sorted[w];
     const int step = gridDim.x * (kOpThreads / 32);
     for (int s = blockIdx.x * (kOpThreads / 32) + w; s < nsl; s += step) {
         const int row = 32 * s + lane, b = __ldg(base + s), steps = __ldg(base + s + 1) - b;
@@ -131,8 +134,6 @@ __global__ void __launch_bounds__(kOpThreads) k_outer_slices(int n, int nsl, con
             d = __ldg(diag + row);
             m = __ldg(mu + row);
         }
-        const bool small = cnt <= kFlatCap;
-        double2 *out = small ? sorted[w] : g + k0;
         for (int u0 = 0; u0 < steps; u0 += kOpGroup) {
             int c[kOpGroup];
             double2 xv[kOpGroup];
@@ -151,17 +152,9 @@ __global__ void __launch_bounds__(kOpThreads) k_outer_slices(int n, int nsl, con
                 if (c[q] >= 0) out[beg + e] = v;
             }
         }
-        for (unsigned lm = longs ? __ldg(longs + s) : 0u; lm; lm &= lm - 1) {   // long rows: from the CSR arrays
-            const int l = __ffs(lm) - 1, e = __ldg(rowptr + 32 * s + l + 1);
-            const double2 ml = __ldg(mu + 32 * s + l);
-            for (int k = __ldg(rowptr + 32 * s + l) + lane; k < e; k += 32)
-                out[k - k0] = neg_conj_mul(ml, __ldg(x + __ldg(col + k)));
-        }
-        if (small) {
-            __syncwarp();
-            for (int i = lane; i < cnt; i += 32) g[k0 + i] = sorted[w][i];
-            __syncwarp();
-        }
+        __syncwarp();
+        for (int i = lane; i < cnt; i += 32) g[k0 + i] = out[i];
+        __syncwarp();
     }
 }
 
@@ -216,13 +209,13 @@ extern "C" HZ_API hz_status hz_outer_on_pattern(const hz_mat *A, const hz_z *d_m
     HZ_CHECK(A, "hz_outer_on_pattern: null handle");
     if (A->n == 0 || A->nnz == 0) return HZ_OK;
     HZ_CHECK(d_mu && d_x && d_gradval, "hz_outer_on_pattern: null vector");
-    if (A->nsl) {
+    if (A->nsl && !A->sl_long && A->sl_most <= kOpSliceCap) {
         DevInfo d;
         HZ_TRY(dev_info(&d));
         const int grid = (int)std::max<int64_t>(
             1, std::min<int64_t>((A->nsl + kOpThreads / 32 - 1) / (kOpThreads / 32), (int64_t)d.num_sms * 16));
         k_outer_slices<<<grid, kOpThreads, 0, (cudaStream_t)stream>>>(A->n, A->nsl, A->sl_base, A->sl_diag, A->sl_col,
-                                                                      A->rowptr, A->sl_long, A->col, (const double2 *)d_mu,
+                                                                      A->rowptr, (const double2 *)d_mu,
                                                                       (const double2 *)d_x, (double2 *)d_gradval);
         HZ_CUDA(cudaGetLastError());
         return HZ_OK;

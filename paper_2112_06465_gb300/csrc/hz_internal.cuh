@@ -641,6 +641,7 @@ struct hz_mat {
     void *sl_mem = nullptr;        // the arrays below but sl_val32
     int32_t *sl_base = nullptr;    // [nsl + 1]
     std::vector<int32_t> sl_base_h;   // the same on the host
+    int32_t sl_most = 0;           // entries of the fullest slice
     uint64_t *sl_mask = nullptr;   // [nsl]
     int32_t *sl_diag = nullptr;    // [n] place of the diagonal entry in its row (-1: absent)
     int32_t *sl_col = nullptr;     // [sl_slots]

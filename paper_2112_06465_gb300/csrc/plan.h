@@ -34,6 +34,7 @@ struct SlicePlan {
     std::vector<unsigned> longs;   // [slices] lanes of long rows
     int64_t slots = 0;
     int64_t nlong = 0;
+    int32_t most = 0;              // entries of the fullest slice
 };
 
 // Padded rows cost binary64 instructions, so the padded size may exceed the
@@ -77,6 +78,7 @@ inline SlicePlan slice_plan(const int32_t *rp, int32_t n, int32_t nnz) {
             }
         }
         p.base[q] = (int32_t)std::min<int64_t>(P, INT32_MAX);
+        p.most = std::max(p.most, rp[std::min(n, 32 * q + 32)] - rp[32 * q]);
         P += w;
         wmax = std::max(wmax, w);
         passes_max = std::max(passes_max, passes);

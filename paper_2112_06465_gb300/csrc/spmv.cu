@@ -655,6 +655,7 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
             A->nsl = ns;
             A->sl_slots = slots;
             A->sl_base_h = sp.base;
+            A->sl_most = sp.most;
             // one allocation (creation is paid for by every new operator)
             const size_t bytes[7] = {sizeof(double) * slots, sizeof(double) * slots, sizeof(uint64_t) * ns,
                                      sizeof(int) * slots,    sizeof(int) * n,        sizeof(int) * (ns + 1),

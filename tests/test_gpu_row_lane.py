@@ -207,3 +207,19 @@ def test_long_rows_together(hz, oracle, count, length, slices):
     err = np.abs(host(hz.cspmv(M, dev(x32))) - oracle.cspmv(A, x32))
     assert np.all(err <= bound(A, x32.astype(np.complex128), 2.0 ** -23))
     M.close()
+
+
+@pytest.mark.parametrize("n,width,diag", [
+    (1, 1, "all"), (33, 7, "all"), (1000, 7, "some"), (1000, 8, "twice"), (1000, 9, "some"), (777, 27, "some"),
+    (777, 27, "twice")])
+def test_outer_product_rows(hz, n, width, diag):
+    """The outer product on slices of up to 256 entries and on the row blocks:
+    rows without a diagonal entry or without any, a diagonal stored twice."""
+    A = banded(n, width, 5 * n + width, diag=diag)
+    mu, x = K.vectors(n, 21)
+    M = hz.Matrix.from_csr(A)
+    g = host(hz.outer_on_pattern(M, dev(mu), dev(x)))
+    rows = np.repeat(np.arange(n), np.diff(A.rowptr))
+    # two products and a sum per component
+    assert np.all(np.abs(g + np.conj(mu[rows] * x[A.col])) <= 4 * 2.0 ** -53 * np.abs(mu[rows]) * np.abs(x[A.col]))
+    M.close()
