@@ -680,7 +680,7 @@ static hz_status get_solver(hz_mat *A, uint32_t mode, cudaStream_t s, Solver **o
             // at once: a grid sized for another epilogue's instantiation
             // would run a partial second wave if these held more registers
             int o1 = 0, o2 = 0;
-            const bool sl = A->nsl && A->sl_val32;
+            const bool sl = A->sl_val32 && A->sl_prod32;
             const cudaError_t e1 =
                 sl ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_spmv_sl<float2, EpiSigma<float2>>, kFlatThreads, 0)
                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_spmv_c64b<EpiSigma<float2>>, kFlatThreads, 0);

@@ -642,6 +642,7 @@ struct hz_mat {
     int32_t *sl_base = nullptr;    // [nsl + 1]
     std::vector<int32_t> sl_base_h;   // the same on the host
     int32_t sl_most = 0;           // entries of the fullest slice
+    bool sl_prod64 = false, sl_prod32 = false;   // products by themselves read the slices
     uint64_t *sl_mask = nullptr;   // [nsl]
     int32_t *sl_diag = nullptr;    // [n] place of the diagonal entry in its row (-1: absent)
     int32_t *sl_col = nullptr;     // [sl_slots]

@@ -1,5 +1,7 @@
 // plan.h -- decisions of the host side that need no device: which matrices get
-// the row-per-lane layout.  Plain C++, so that a test compiles it by itself.
+// the row-per-lane layout,
+// and which products read it.  Plain
+// C++, so that a test compiles it by itself.
 #pragma once
 
 #include <algorithm>
@@ -35,6 +37,7 @@ struct SlicePlan {
     int64_t slots = 0;
     int64_t nlong = 0;
     int32_t most = 0;              // entries of the fullest slice
+    int32_t width = 0;             // steps of the widest slice
 };
 
 // Padded rows cost binary64 instructions, so the padded size may exceed the
@@ -53,7 +56,7 @@ inline SlicePlan slice_plan(const int32_t *rp, int32_t n, int32_t nnz) {
     p.longs.assign(ns, 0u);
     const double lim = std::max((double)kSlLongRow, 2.0 * ((double)nnz / n));
     int64_t P = 0, short_nnz = nnz;
-    int wmax = 0, rmax = 0, passes_max = 0;
+    int rmax = 0, passes_max = 0;
     for (int q = 0; q < ns; ++q) {
         const int r0 = 32 * q, r1 = std::min(n, r0 + 32);
         int w = 0, passes = 0;
@@ -80,15 +83,35 @@ inline SlicePlan slice_plan(const int32_t *rp, int32_t n, int32_t nnz) {
         p.base[q] = (int32_t)std::min<int64_t>(P, INT32_MAX);
         p.most = std::max(p.most, rp[std::min(n, 32 * q + 32)] - rp[32 * q]);
         P += w;
-        wmax = std::max(wmax, w);
+        p.width = std::max(p.width, w);
         passes_max = std::max(passes_max, passes);
     }
     p.base[ns] = (int32_t)std::min<int64_t>(P, INT32_MAX);
     p.slots = 32 * P;
-    p.fits = P > 0 && wmax <= kSlMaxWidth && rmax <= kSlMaxRow && 128 * p.nlong <= n && passes_max <= kSlLongPasses &&
+    p.fits = P > 0 && p.width <= kSlMaxWidth && rmax <= kSlMaxRow && 128 * p.nlong <= n && passes_max <= kSlLongPasses &&
              p.slots < INT32_MAX - 32 &&
              (4 * p.slots <= 5 * short_nnz || (n <= 65536 && 5 * p.slots <= 7 * short_nnz));
     return p;
+}
+
+// Whether a product by itself reads the slices (the solves on chip always do).
+// A slice is one warp's serial walk over its width, so where there are few of
+// them and they are wide, the row blocks, which spread every row over a warp's
+// lanes, are faster: binary64 on the caller's arrays, complex64 on its copy.
+// us a product, warm, row blocks / slices:
+//   rows of           60          40          27      30 to 60
+//   binary64
+//     4,000       6.6 / 11.7   6.7 / 8.9  10.3 / 7.0   9.1 / 12.1
+//    10,000       9.6 / 12.7   9.2 / 8.9  10.5 / 7.2  11.5 / 12.6
+//    14,000      10.1 / 12.9       - / 9.1     - / 7.0  14.4 / 12.8
+//    24,000      16.8 / 13.9  13.9 / 9.8  16.1 / 7.9  17.9 / 14.0
+//   complex64
+//     4,000       5.4 / 6.7    5.5 / 5.3   5.1 / 4.7   5.8 / 7.1
+//    24,000       6.6 / 8.2    6.5 / 5.8   5.7 / 5.1   6.6 / 8.2
+//    64,000      12.2 / 10.5  12.2 / 7.6   6.6 / 6.0  11.7 / 10.4
+inline bool slice_product(int nsl, int width, bool binary64, int num_sms) {
+    if (binary64) return !((width >= 40 && 2 * nsl <= 3 * num_sms) || (width > 52 && 2 * nsl <= 5 * num_sms));
+    return !(width > 40 && nsl <= 5 * num_sms);
 }
 
 }  // namespace hz

@@ -277,7 +277,7 @@ MatView<double2> mat_view<double2>(const hz_mat *A) {
     v.perm = A->sell_perm; v.scol = A->sell_col; v.sval = A->sell_val;
     v.pk_base = A->pk_base; v.pk_gbase = A->pk_gbase; v.pk_gim = A->pk_gim; v.pk_col = A->pk_col;
     v.pk_re = A->pk_re; v.pk_im = A->pk_im;
-    v.nsl = A->nsl; v.sl_base = A->sl_base; v.sl_mask = (const unsigned long long *)A->sl_mask;
+    v.nsl = A->nsl; v.sl_prod = A->sl_prod64; v.sl_base = A->sl_base; v.sl_mask = (const unsigned long long *)A->sl_mask;
     v.sl_col = A->sl_col; v.sl_re = A->sl_re; v.sl_im = A->sl_im; v.sl_long = A->sl_long;
     return v;
 }
@@ -289,7 +289,7 @@ MatView<float2> mat_view<float2>(const hz_mat *A) {
     v.nfblk = A->nfblk; v.fblk = A->fblk; v.fblk_k = A->fblk_k;
     v.nchunks = A->sell_nchunks; v.chunk_off = A->sell_chunk_off; v.chunk_w = A->sell_chunk_w;
     v.perm = A->sell_perm; v.scol = A->sell_col; v.sval = A->sell_val32;
-    v.nsl = A->sl_val32 ? A->nsl : 0; v.sl_base = A->sl_base; v.sl_col = A->sl_col; v.sl_val32 = A->sl_val32; v.sl_long = A->sl_long;
+    v.nsl = A->sl_val32 ? A->nsl : 0; v.sl_prod = A->sl_val32 && A->sl_prod32; v.sl_base = A->sl_base; v.sl_col = A->sl_col; v.sl_val32 = A->sl_val32; v.sl_long = A->sl_long;
     return v;
 }
 
@@ -300,6 +300,7 @@ int spmv_grid(const hz_mat *A, int kind, int group, int blocks_per_sm_cap) {
         // persistent: exactly the CTAs that fit at once (blocks are taken
         // grid-stride, so CTAs beyond one wave would only add a tail)
         static int occ_flat = 0, occ_tma = 0, occ_d64 = 0, occ_d64p = 0, occ_sl = 0;
+        if (kind == HZ_SPMV_FLAT64P && A->nsl && !A->sl_prod64) kind = HZ_SPMV_FLAT64;
         const bool sl = kind == HZ_SPMV_FLAT64P && A->nsl;
         int &occ = sl ? occ_sl
                    : kind == HZ_SPMV_FF_TMA ? occ_tma
@@ -340,7 +341,7 @@ int spmv_grid(const hz_mat *A, int kind, int group, int blocks_per_sm_cap) {
 int c64_flat_grid(const hz_mat *A) {
     DevInfo d;
     if (dev_info(&d) != HZ_OK) return 1;
-    if (A->nsl && A->sl_val32) {
+    if (A->sl_val32 && A->sl_prod32) {
         static int occ_sl = 0;
         if (occ_sl == 0 &&
             (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_sl, k_spmv_sl<float2, EpiStore<float2>>, kFlatThreads,
@@ -656,6 +657,10 @@ extern "C" HZ_API hz_status hz_csr_create(hz_mat **out, int32_t n, int32_t nnz, 
             A->sl_slots = slots;
             A->sl_base_h = sp.base;
             A->sl_most = sp.most;
+            DevInfo d;
+            if (dev_info(&d) != HZ_OK) return fail(HZ_ERR_CUDA);
+            A->sl_prod64 = slice_product(ns, sp.width, true, d.num_sms);
+            A->sl_prod32 = slice_product(ns, sp.width, false, d.num_sms);
             // one allocation (creation is paid for by every new operator)
             const size_t bytes[7] = {sizeof(double) * slots, sizeof(double) * slots, sizeof(uint64_t) * ns,
                                      sizeof(int) * slots,    sizeof(int) * n,        sizeof(int) * (ns + 1),

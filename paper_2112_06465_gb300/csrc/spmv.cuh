@@ -112,6 +112,7 @@ struct MatView {
     const double *pk_im;
     // row-per-lane stream (see hz_mat::sl_*); nsl = 0 without it
     int nsl;
+    bool sl_prod;   // products by themselves read it (slice_product)
     const int *sl_base;
     const unsigned long long *sl_mask;
     const int *sl_col;
@@ -1558,7 +1559,7 @@ cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, cudaS
 template <class Epi>
 cudaError_t launch_c64_flat(bool pdl, int grid, const MatView<float2> &A, const float2 *x, const Epi &epi,
                             RedScratch red, cudaStream_t s) {
-    if (A.nsl) return launch_k(pdl, k_spmv_sl<float2, Epi>, grid, kFlatThreads, s, A, x, epi, red);
+    if (A.sl_prod) return launch_k(pdl, k_spmv_sl<float2, Epi>, grid, kFlatThreads, s, A, x, epi, red);
     return launch_k(pdl, k_spmv_c64b<Epi>, grid, kFlatThreads, s, A, x, epi, red);
 }
 
@@ -1567,7 +1568,7 @@ template <class T, class Epi>
 cudaError_t launch_spmv(int kind, int group, const MatView<T> &A, const T *x, const Epi &epi,
                         RedScratch red, int grid, cudaStream_t s, bool pdl = false) {
     if constexpr (std::is_same<T, double2>::value) {
-        if (kind == HZ_SPMV_FLAT64) {
+        if (kind == HZ_SPMV_FLAT64 || (kind == HZ_SPMV_FLAT64P && A.nsl && !A.sl_prod)) {
             launch_k(pdl, k_spmv_d64b<Epi, false>, grid, kFlatThreads, s, A, x, epi, red);
             return cudaGetLastError();
         }

@@ -223,3 +223,28 @@ def test_outer_product_rows(hz, n, width, diag):
     # two products and a sum per component
     assert np.all(np.abs(g + np.conj(mu[rows] * x[A.col])) <= 4 * 2.0 ** -53 * np.abs(mu[rows]) * np.abs(x[A.col]))
     M.close()
+
+
+@pytest.mark.parametrize("slices_per_sm,width,slices", [
+    (1.0, 39, True), (1.0, 40, False), (1.5, 40, False), (1.52, 40, True), (2.5, 52, True), (2.5, 53, False),
+    (2.52, 53, True), (5.0, 41, True)])
+def test_few_wide_slices(hz, oracle, slices_per_sm, width, slices):
+    """A product by itself reads the row blocks where the slices are few and
+    wide (complex64: above 40 steps up to 5 slices per SM); a solve on chip of
+    the same handle reads the slices."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 32 * int(np.ceil(slices_per_sm * sms) if slices else slices_per_sm * sms)
+    A = banded(n, width, width, real=False)
+    A.val[A.col == np.repeat(np.arange(n), np.diff(A.rowptr))] += 4.0 * width   # (for the solve)
+    x = K.vectors(n, 23)[0]
+    assert on_slices(hz, A, x) == slices
+    M = hz.Matrix.from_csr(A, c64=True)
+    assert np.all(np.abs(host(hz.zspmv(M, dev(x))) - oracle.zspmv(A, x)) <= bound(A, x))
+    x32 = x.astype(np.complex64)
+    err = np.abs(host(hz.cspmv(M, dev(x32))) - oracle.cspmv(A, x32))
+    assert np.all(err <= bound(A, x32.astype(np.complex128), 2.0 ** -23))
+    for kw in (dict(), dict(mode="mixed"), dict(method="bicgstabl")):
+        y, info = hz.zsolve(M, dev(x), tol=1e-11, maxit=100, **kw)
+        assert info.status == 0
+        assert np.linalg.norm(x - oracle.zspmv(A, host(y))) <= 2e-11 * np.linalg.norm(x)
+    M.close()

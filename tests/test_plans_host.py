@@ -1,5 +1,5 @@
 """Host decisions of csrc/plan.h, compiled by themselves: the row-per-lane
-layout."""
+layout and the products that read it."""
 
 import ctypes as C
 import os
@@ -20,6 +20,7 @@ extern "C" int slices(const int *rp, int n, int *base, unsigned *longs, long lon
     *slots = p.slots;
     return p.fits;
 }
+extern "C" int product(int nsl, int width, int binary64, int sms) { return slice_product(nsl, width, binary64, sms); }
 """
 
 
@@ -86,3 +87,13 @@ def test_long_rows_that_lie_together(plan, count, length, fits):
     lens = np.full(8000, 7)
     lens[:64 * 63:64] = 100            # more than one row in 128
     assert not slices(plan, lens)[0]
+
+
+def test_products_of_few_wide_slices(plan):
+    """Edges of the rule on 152 SMs: which products by themselves read the slices."""
+    f = lambda nsl, width, b64: bool(plan.product(nsl, width, b64, 152))
+    assert all(f(nsl, w, 1) for nsl in (1, 100, 100000) for w in (1, 15, 39))
+    assert [f(nsl, 40, 1) for nsl in (1, 228, 229, 380, 381)] == [False, False, True, True, True]
+    assert [f(nsl, 53, 1) for nsl in (1, 228, 229, 380, 381)] == [False, False, False, False, True]
+    assert [f(nsl, 40, 0) for nsl in (1, 760)] == [True, True]
+    assert [f(nsl, 41, 0) for nsl in (1, 760, 761)] == [False, False, True]
