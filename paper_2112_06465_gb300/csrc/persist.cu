@@ -1255,36 +1255,13 @@ void ps_batch_free(void *p) {
 bool ps_batch_plan(hz_mat *const *A, int ns, std::vector<int> *ncta) {
     DevInfo d;
     if (dev_info(&d) != HZ_OK) return false;
-    ncta->assign(ns, 0);
-    int64_t total = 0;
+    std::vector<int> nsl(ns, 0);
     for (int k = 0; k < ns; ++k) {
         if (A[k]->n == 0) continue;
         if (!ps_layout(A[k])) return false;
-        total += A[k]->nsl;
+        nsl[k] = A[k]->nsl;
     }
-    int left = d.num_sms;
-    for (int k = 0; k < ns; ++k) {
-        if (A[k]->n == 0) continue;
-        const int cap = std::min(A[k]->nsl, kPsMaxCta);
-        (*ncta)[k] = std::max(1, std::min(cap, (int)((int64_t)d.num_sms * A[k]->nsl / total)));
-        left -= (*ncta)[k];
-    }
-    if (left < 0) return false;   // more small systems than CTAs
-    for (; left > 0; --left) {
-        int best = -1;
-        double most = 0.0;
-        for (int k = 0; k < ns; ++k) {
-            const int c = (*ncta)[k];
-            if (c == 0 || c >= std::min(A[k]->nsl, kPsMaxCta)) continue;
-            const double load = (double)A[k]->nsl / c;
-            if (load > most) { most = load; best = k; }
-        }
-        if (best < 0) break;
-        (*ncta)[best] += 1;
-    }
-    for (int k = 0; k < ns; ++k)
-        if ((*ncta)[k] && (A[k]->nsl + (*ncta)[k] - 1) / (*ncta)[k] > ps_slices(PS_BICG)) return false;
-    return true;
+    return sweep_plan(nsl, d.num_sms, kPsMaxCta, ps_slices(PS_BICG), ncta);
 }
 
 hz_status ps_solve_batched(hz_mat *const *A, int ns, const std::vector<int> &ncta, const double2 *const *b,

@@ -1,6 +1,6 @@
 // plan.h -- decisions of the host side that need no device: which matrices get
 // the row-per-lane layout,
-// and which products read it.  Plain
+// which products read it, and how a sweep shares the SMs.  Plain
 // C++, so that a test compiles it by itself.
 #pragma once
 
@@ -112,6 +112,54 @@ inline SlicePlan slice_plan(const int32_t *rp, int32_t n, int32_t nnz) {
 inline bool slice_product(int nsl, int width, bool binary64, int num_sms) {
     if (binary64) return !((width >= 40 && 2 * nsl <= 3 * num_sms) || (width > 52 && 2 * nsl <= 5 * num_sms));
     return !(width > 40 && nsl <= 5 * num_sms);
+}
+
+// The CTAs of each system of a sweep on chip, one CTA per SM: nsl slices each
+// (0: an empty system, no CTA), at most max_cta CTAs a system and max_slices
+// slices a CTA.  Shares by slices, then one CTA more at a time to the system
+// whose CTAs own the most; where rounding the small shares up to one CTA and
+// the others down leaves too few, every system starts from one.  False where
+// they do not fit.
+// us per iteration of the slowest system, in the grid-wide phases / on chip,
+// all systems running (rows of 7, 15 and 27 entries):
+//   64,000 unknowns with 100 boxes of 1,000    146 / 58   179 / 84   259 / 116
+//   125,000 unknowns with 80 boxes of 1,000    146 / 66   182 / 104  263 / 151
+inline bool sweep_plan(const std::vector<int> &nsl, int num_sms, int max_cta, int max_slices, std::vector<int> *ncta) {
+    const int ns = (int)nsl.size();
+    std::vector<int> &c = *ncta;
+    int64_t total = 0;
+    int live = 0;
+    for (int n : nsl) {
+        total += n;
+        live += n > 0;
+    }
+    c.assign(ns, 0);
+    if (live > num_sms) return false;
+    auto cap = [&](int k) { return std::min(nsl[k], max_cta); };
+    for (int start = 0; start < 2; ++start) {
+        int left = num_sms;
+        for (int k = 0; k < ns; ++k) {
+            if (nsl[k] == 0) continue;
+            c[k] = start ? 1 : std::max(1, std::min(cap(k), (int)((int64_t)num_sms * nsl[k] / total)));
+            left -= c[k];
+        }
+        if (left < 0) continue;
+        for (; left > 0; --left) {
+            int best = -1;
+            double most = 0.0;
+            for (int k = 0; k < ns; ++k) {
+                if (c[k] == 0 || c[k] >= cap(k)) continue;
+                const double load = (double)nsl[k] / c[k];
+                if (load > most) { most = load; best = k; }
+            }
+            if (best < 0) break;
+            c[best] += 1;
+        }
+        bool ok = true;
+        for (int k = 0; k < ns; ++k) ok = ok && (c[k] == 0 || (nsl[k] + c[k] - 1) / c[k] <= max_slices);
+        if (ok) return true;
+    }
+    return false;
 }
 
 }  // namespace hz

@@ -227,3 +227,45 @@ def test_threads_sweep_the_same_handles(hz):
     alone, _ = hz.zsolve_batched(mats, bs, tol=TOL, maxit=200)
     for o in out:
         assert len(o) == 20 and all(torch.equal(x, y) for xs in o for x, y in zip(xs, alone))
+
+
+def unlike_the_graph(hz, mats, bs, x0s):
+    """(solutions of a sweep, whether it ran on chip): the grid-wide phases give
+    handles of either binary64 kind the same sums, a sweep on chip other ones."""
+    out = []
+    for kind in ("flat64p", "flat64"):
+        for M in mats:
+            M.set_spmv(kind)
+        out.append(hz.zsolve_batched(mats, bs, xs=[x.clone() for x in x0s], tol=TOL, maxit=200))
+    (xa, ia), (xb, _) = out
+    for M in mats:
+        M.set_spmv("flat64p")
+    return xa, ia, not all(torch.equal(p, q) for p, q in zip(xa, xb))
+
+
+@pytest.mark.parametrize("sizes,chip", [
+    ((20011, 31, 4865, 700, 300), True),         # shares of 1 to 117 CTAs
+    ((4865,) + (31,) * 140, True),               # small systems rounded up to one CTA each
+    ((700,) * 151 + (1000,), True),              # one CTA each
+    ((4865,) + (31,) * 152, False),              # more systems than SMs
+    ((20011,) + (31,) * 150, False),             # two CTAs cannot hold the large one
+    ((33, 20011, 1, 700), False)])               # padding keeps two of them off the layout
+def test_sweep_shares(hz, sizes, chip):
+    """Uneven sweeps: which of them run on chip, and every system against its
+    single solve, from a start vector, a zero right-hand side among them."""
+    mats = [hz.Matrix.from_csr(operator(n, 7 + k)) for k, n in enumerate(sizes)]
+    bs = [vec(n, 50 + k) for k, n in enumerate(sizes)]
+    x0s = [vec(n, 300 + k) for k, n in enumerate(sizes)]
+    bs[3].zero_()
+    xs, infos, on_chip = unlike_the_graph(hz, mats, bs, x0s)
+    assert on_chip == chip
+    for k, (M, b, x, info) in enumerate(zip(mats, bs, xs, infos)):
+        assert info.status == 0, (k, info)
+        if k == 3:
+            assert info.iters == 0 and torch.equal(x, x0s[3])
+        elif k < 6:
+            y, one = hz.zsolve(M, b, x=x0s[k].clone(), tol=TOL, maxit=200)
+            assert float(torch.linalg.vector_norm(x - y) / torch.linalg.vector_norm(y)) <= 3.5 * TOL
+            assert abs(info.iters - one.iters) <= 2 + one.iters // 4
+    for M in mats:
+        M.close()

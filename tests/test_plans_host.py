@@ -1,5 +1,5 @@
 """Host decisions of csrc/plan.h, compiled by themselves: the row-per-lane
-layout and the products that read it."""
+layout, the products that read it and the SMs of a sweep's systems."""
 
 import ctypes as C
 import os
@@ -21,6 +21,12 @@ extern "C" int slices(const int *rp, int n, int *base, unsigned *longs, long lon
     return p.fits;
 }
 extern "C" int product(int nsl, int width, int binary64, int sms) { return slice_product(nsl, width, binary64, sms); }
+extern "C" int sweep(int ns, const int *nsl, int sms, int max_cta, int max_slices, int *ncta) {
+    std::vector<int> c;
+    const bool ok = sweep_plan(std::vector<int>(nsl, nsl + ns), sms, max_cta, max_slices, &c);
+    std::copy(c.begin(), c.end(), ncta);
+    return ok;
+}
 """
 
 
@@ -97,3 +103,31 @@ def test_products_of_few_wide_slices(plan):
     assert [f(nsl, 53, 1) for nsl in (1, 228, 229, 380, 381)] == [False, False, False, False, True]
     assert [f(nsl, 40, 0) for nsl in (1, 760)] == [True, True]
     assert [f(nsl, 41, 0) for nsl in (1, 760, 761)] == [False, False, True]
+
+
+def shares(plan, nsl, sms=152, max_cta=160, max_slices=60):
+    a, out = np.array(nsl, np.int32), np.zeros(len(nsl), np.int32)
+    ok = plan.sweep(len(nsl), a.ctypes.data_as(C.c_void_p), sms, max_cta, max_slices, out.ctypes.data_as(C.c_void_p))
+    return bool(ok), [int(c) for c in out]
+
+
+@pytest.mark.parametrize("nsl,fits", [
+    ([2000] + [32] * 100, True), ([1500] + [10] * 60, True), ([2, 626, 1, 22], True), ([626, 1, 153, 22, 10], True),
+    ([32] * 152, True), ([32] * 153, False), ([626] + [1] * 150, False), ([153] + [1] * 140, True),
+    ([9121], False), ([9120], True), ([0, 5, 0, 9], True), ([7628] + [61] * 12, True), ([0, 0], True), ([1], True)])
+def test_sweep_shares(plan, nsl, fits):
+    """A sweep runs on chip exactly where one CTA for each system and enough
+    for the large ones fit on the SMs together; then no SM stays idle that a
+    system could use, and no CTA holds more than its slices."""
+    ok, c = shares(plan, nsl)
+    assert ok == fits == (sum(-(-n // 60) for n in nsl) <= 152)
+    if not ok:
+        return
+    assert sum(c) <= 152 and all((n > 0) == (k > 0) and k <= n for n, k in zip(nsl, c))
+    assert sum(c) == 152 or all(k == n for n, k in zip(nsl, c))
+    assert all(-(-n // k) <= 60 for n, k in zip(nsl, c) if k)
+
+
+def test_sweep_shares_of_even_systems(plan):
+    assert shares(plan, [100, 100, 100, 100]) == (True, [38, 38, 38, 38])
+    assert shares(plan, [432, 432, 106, 106], sms=100) == (True, [40, 40, 10, 10])
