@@ -842,10 +842,11 @@ extern "C" HZ_API hz_status hz_zsolve_batched(int32_t nsys, hz_mat *const *A, co
         for (int k = 0; k < nsys; ++k)
             HZ_CHECK(A[k]->n == 0 || (d_b[k] && d_x[k]), "hz_zsolve_batched: null vector");
         std::vector<Info> inf(nsys);
+        bool taken = false;
         HZ_TRY(ps_solve_batched(A, nsys, ncta, (const double2 *const *)d_b, (double2 *const *)d_x, tol, maxit,
-                                inf.data(), s));
+                                inf.data(), s, &taken));
         hz_status worst = HZ_OK;
-        for (int k = 0; k < nsys; ++k) {
+        for (int k = 0; taken && k < nsys; ++k) {
             hz_info &o = h_info[k];
             o = hz_info{};
             o.iters = inf[k].iters;
@@ -855,7 +856,7 @@ extern "C" HZ_API hz_status hz_zsolve_batched(int32_t nsys, hz_mat *const *A, co
             if (o.status == HZ_OK && o.relres_true > tol) o.status = HZ_NOT_CONVERGED;
             if (o.status != HZ_OK && worst == HZ_OK) worst = (hz_status)o.status;
         }
-        return worst;
+        if (taken) return worst;
     }
     // per system: 16-byte vectors (6 binary64 or 7 double-float; mixed: the
     // best iterate) and, in a mixed batch, 7 complex64 inner vectors

@@ -755,38 +755,36 @@ extern "C" HZ_API hz_status hz_zsolve_opts(hz_mat *A, const hz_z *d_b, hz_z *d_x
     c.op_scale = 1.0;
     // systems whose vectors fit on chip: one persistent kernel
     const PsKind pk = o->method == HZ_METHOD_TFQMR ? PS_TFQMR : o->mode == HZ_MODE_MIXED ? PS_MIXED : PS_BICG;
-    const bool ps = o->method != HZ_METHOD_BICGSTABL && ps_fits(op, pk);
-    if (ps || o->method == HZ_METHOD_BICGSTABL || o->method == HZ_METHOD_TFQMR) {
-        Info inf{};
-        int restarts = 0;
-        if (ps) {
-            if (pk == PS_MIXED) HZ_TRY(ensure_c64(op, s));
-            HZ_TRY(ps_solve(op, pk, c, &inf, &restarts, s));
-        } else if (o->method == HZ_METHOD_BICGSTABL) HZ_TRY(bl_solve(op, o->ell, c, &inf, &restarts, s));
-        else HZ_TRY(tq_solve(op, c, &inf, &restarts, s));
-        if (inf.status == HZ_OK && inf.relres_true > o->tol) inf.status = HZ_NOT_CONVERGED;
-        h_info->iters = inf.iters;
-        h_info->status = inf.status;
-        h_info->restarts = restarts;
-        h_info->outer = inf.outer;
-        h_info->relres_rec = inf.relres_rec;
-        h_info->relres_true = inf.relres_true;
-        return (hz_status)inf.status;
-    }
-    Solver *S = nullptr;
-    HZ_TRY(get_solver(op, o->mode, s, &S));
-    *S->hctl = c;
-    S->hctl->op_scale = S->op_scale;
-    HZ_CUDA(cudaGraphLaunch(S->exec, s));
-    HZ_CUDA(cudaStreamSynchronize(s));
-    Info inf = *S->hinfo;
+    Info inf{};
     int restarts = 0;
-    if (o->mode == HZ_MODE_FP64 && inf.status == HZ_OK && inf.relres_true > o->tol && inf.iters < o->maxit) {
-        S->hctl->restart = 1;
-        restarts = 1;
+    bool done = false;
+    if (o->method != HZ_METHOD_BICGSTABL && ps_fits(op, pk)) {
+        if (pk == PS_MIXED) HZ_TRY(ensure_c64(op, s));
+        HZ_TRY(ps_solve(op, pk, c, &inf, &restarts, s, &done));
+    }
+    if (!done && o->method == HZ_METHOD_BICGSTABL) {
+        HZ_TRY(bl_solve(op, o->ell, c, &inf, &restarts, s));
+        done = true;
+    }
+    if (!done && o->method == HZ_METHOD_TFQMR) {
+        HZ_TRY(tq_solve(op, c, &inf, &restarts, s));
+        done = true;
+    }
+    if (!done) {
+        Solver *S = nullptr;
+        HZ_TRY(get_solver(op, o->mode, s, &S));
+        *S->hctl = c;
+        S->hctl->op_scale = S->op_scale;
         HZ_CUDA(cudaGraphLaunch(S->exec, s));
         HZ_CUDA(cudaStreamSynchronize(s));
         inf = *S->hinfo;
+        if (o->mode == HZ_MODE_FP64 && inf.status == HZ_OK && inf.relres_true > o->tol && inf.iters < o->maxit) {
+            S->hctl->restart = 1;
+            restarts = 1;
+            HZ_CUDA(cudaGraphLaunch(S->exec, s));
+            HZ_CUDA(cudaStreamSynchronize(s));
+            inf = *S->hinfo;
+        }
     }
     if (inf.status == HZ_OK && inf.relres_true > o->tol) inf.status = HZ_NOT_CONVERGED;
     h_info->iters = inf.iters;

@@ -1113,7 +1113,9 @@ static int ps_cluster(const hz_mat *A, PsKind kind, size_t *smem) {
     return *smem <= (size_t)kPsSmem ? c : 0;
 }
 
-static cudaError_t ps_launch_cluster(PsKind kind, int ctas, int slices, size_t smem, PsSys *dsys, cudaStream_t s) {
+// (clusters: how many the device holds at once, asked for at -1)
+static cudaError_t ps_launch_cluster(PsKind kind, int ctas, int slices, size_t smem, PsSys *dsys, cudaStream_t s,
+                                     int *clusters) {
     void *kern = ps_method(kind).kern[2];
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPsSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1131,13 +1133,25 @@ static cudaError_t ps_launch_cluster(PsKind kind, int ctas, int slices, size_t s
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    if (*clusters < 0) {
+        e = cudaOccupancyMaxActiveClusters(clusters, kern, &cfg);
+        if (e != cudaSuccess) { *clusters = -1; return e; }
+    }
+    if (*clusters == 0) return cudaErrorLaunchOutOfResources;
     int ns = 1;
     void *args[] = {&dsys, &ns};
     return cudaLaunchKernelExC(&cfg, kern, args);
 }
 
+// what a launch says that the device has no room for (nothing ran; not sticky)
+static bool ps_no_room(cudaError_t e) {
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+           e == cudaErrorInvalidClusterSize || e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported;
+}
+
 struct PsSolver {
     int n = 0;
+    int clusters = -1;         // clusters of its size that the device holds (-1: not asked)
     void *mem = nullptr;       // lines, err, info, system, vectors
     PsSys *dsys = nullptr;
     Info *dinfo = nullptr;
@@ -1193,7 +1207,8 @@ static hz_status ps_get(hz_mat *A, PsKind kind, PsSolver **out) {
     return HZ_OK;
 }
 
-hz_status ps_solve(hz_mat *A, PsKind kind, const Ctl &c, Info *out, int *restarts, cudaStream_t s) {
+hz_status ps_solve(hz_mat *A, PsKind kind, const Ctl &c, Info *out, int *restarts, cudaStream_t s, bool *taken) {
+    *taken = true;
     PsSolver *S = nullptr;
     HZ_TRY(ps_get(A, kind, &S));
     DevInfo d;
@@ -1208,13 +1223,29 @@ hz_status ps_solve(hz_mat *A, PsKind kind, const Ctl &c, Info *out, int *restart
     h.cta0 = 0;
     size_t smem = 0;
     const int cl = ps_cluster(A, kind, &smem);
-    h.ncta = cl ? cl : ps_ctas(A, d.num_sms);
+    Way way = cl ? Way::cluster : Way::all_sms;
     *restarts = 0;
     for (int run = 0;; ++run) {
-        HZ_CUDA(cudaMemcpyAsync(S->dsys, &h, sizeof(PsSys), cudaMemcpyHostToDevice, s));
-        HZ_CUDA(cudaMemsetAsync(S->lines, 0, kPsErrOff + sizeof(int), s));
-        HZ_CUDA(cl ? ps_launch_cluster(kind, cl, (A->nsl + cl - 1) / cl, smem, S->dsys, s)
-                   : ps_launch(kind, &A, &h, 1, S->dsys, s));
+        cudaError_t e = cudaSuccess;
+        const bool ok = first_way(way, [&](Way w) {
+            h.ncta = w == Way::cluster ? cl : ps_ctas(A, d.num_sms);
+            e = cudaMemcpyAsync(S->dsys, &h, sizeof(PsSys), cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(S->lines, 0, kPsErrOff + sizeof(int), s);
+            if (e != cudaSuccess) return Launch::error;
+            e = w == Way::cluster ? ps_launch_cluster(kind, cl, (A->nsl + cl - 1) / cl, smem, S->dsys, s, &S->clusters)
+                                  : ps_launch(kind, &A, &h, 1, S->dsys, s);
+            if (e == cudaSuccess) return Launch::done;
+            if (!ps_no_room(e)) return Launch::error;
+            cudaGetLastError();
+            // (h is written again only when the copy above has read it)
+            e = cudaStreamSynchronize(s);
+            return e == cudaSuccess ? Launch::no_room : Launch::error;
+        });
+        if (!ok) return cuda_fail(e, "hz_zsolve", __FILE__, __LINE__);
+        if (way == Way::graph) {
+            if (run == 0) { *taken = false; return HZ_OK; }
+            return cuda_fail(cudaErrorCooperativeLaunchTooLarge, "hz_zsolve (restart)", __FILE__, __LINE__);
+        }
         HZ_CUDA(cudaMemcpyAsync(&S->hback->info, S->dinfo, sizeof(Info), cudaMemcpyDeviceToHost, s));
         HZ_CUDA(cudaMemcpyAsync(&S->hback->err, S->err, sizeof(int), cudaMemcpyDeviceToHost, s));
         HZ_CUDA(cudaStreamSynchronize(s));
@@ -1265,7 +1296,8 @@ bool ps_batch_plan(hz_mat *const *A, int ns, std::vector<int> *ncta) {
 }
 
 hz_status ps_solve_batched(hz_mat *const *A, int ns, const std::vector<int> &ncta, const double2 *const *b,
-                           double2 *const *x, double tol, int maxit, Info *out, cudaStream_t s) {
+                           double2 *const *x, double tol, int maxit, Info *out, cudaStream_t s, bool *taken) {
+    *taken = true;
     std::vector<hz_mat *> act;
     std::vector<int> idx;
     for (int k = 0; k < ns; ++k) {
@@ -1346,7 +1378,14 @@ hz_status ps_solve_batched(hz_mat *const *A, int ns, const std::vector<int> &nct
     int err = 0;
     e = cudaMemsetAsync(mem, 0, zero_b, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dsys, h.data(), sizeof(PsSys) * na, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = ps_launch(PS_BICG, act.data(), h.data(), na, dsys, s);
+    if (e == cudaSuccess) {
+        e = ps_launch(PS_BICG, act.data(), h.data(), na, dsys, s);
+        if (ps_no_room(e)) {   // the caller's phases take the sweep
+            cudaGetLastError();
+            e = cudaSuccess;
+            *taken = false;
+        }
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(hi.data(), mem + 256, sizeof(Info) * na, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, mem, sizeof(int), cudaMemcpyDeviceToHost, s);
     const cudaError_t e2 = cudaStreamSynchronize(s);   // (also after a failure: the workspace is free again)
@@ -1354,6 +1393,7 @@ hz_status ps_solve_batched(hz_mat *const *A, int ns, const std::vector<int> &nct
     if (mine) B->busy.clear(std::memory_order_release);
     else cudaFree(mem);
     if (e != cudaSuccess) return cuda_fail(e, "hz_zsolve_batched", __FILE__, __LINE__);
+    if (!*taken) return HZ_OK;
     if (err) {
         set_error("hz_zsolve_batched: a barrier wait of the persistent solver expired");
         return HZ_ERR_TIMEOUT;

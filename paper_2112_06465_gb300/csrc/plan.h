@@ -1,6 +1,6 @@
 // plan.h -- decisions of the host side that need no device: which matrices get
 // the row-per-lane layout,
-// which products read it, and how a sweep shares the SMs.  Plain
+// which products read it, how a solve runs and how a sweep shares the SMs.  Plain
 // C++, so that a test compiles it by itself.
 #pragma once
 
@@ -112,6 +112,22 @@ inline SlicePlan slice_plan(const int32_t *rp, int32_t n, int32_t nnz) {
 inline bool slice_product(int nsl, int width, bool binary64, int num_sms) {
     if (binary64) return !((width >= 40 && 2 * nsl <= 3 * num_sms) || (width > 52 && 2 * nsl <= 5 * num_sms));
     return !(width > 40 && nsl <= 5 * num_sms);
+}
+
+// How a solve runs, and what it falls back to where the device has no room for
+// a launch (a partition, or a share of the SMs given to other work): one
+// cluster, every SM, the graph of kernels.
+enum class Way { cluster, all_sms, graph };
+enum class Launch { done, no_room, error };
+// launch(way) on the ways from `way` on until one is taken; the graph is the
+// caller's.  True unless a launch failed for another reason.
+template <class F> inline bool first_way(Way &way, F launch) {
+    while (way != Way::graph) {
+        const Launch r = launch(way);
+        if (r != Launch::no_room) return r == Launch::done;
+        way = way == Way::cluster ? Way::all_sms : Way::graph;
+    }
+    return true;
 }
 
 // The CTAs of each system of a sweep on chip, one CTA per SM: nsl slices each

@@ -1,5 +1,6 @@
 """Host decisions of csrc/plan.h, compiled by themselves: the row-per-lane
-layout, the products that read it and the SMs of a sweep's systems."""
+layout, the products that read it, the ways of a solve and the SMs of a sweep's
+systems."""
 
 import ctypes as C
 import os
@@ -25,6 +26,16 @@ extern "C" int sweep(int ns, const int *nsl, int sms, int max_cta, int max_slice
     std::vector<int> c;
     const bool ok = sweep_plan(std::vector<int>(nsl, nsl + ns), sms, max_cta, max_slices, &c);
     std::copy(c.begin(), c.end(), ncta);
+    return ok;
+}
+extern "C" int ways(int *way, const int *answers, int *tried, int *n) {
+    Way w = (Way)*way;
+    *n = 0;
+    const bool ok = first_way(w, [&](Way v) {
+        tried[*n] = (int)v;
+        return (Launch)answers[(*n)++];
+    });
+    *way = (int)w;
     return ok;
 }
 """
@@ -131,3 +142,15 @@ def test_sweep_shares(plan, nsl, fits):
 def test_sweep_shares_of_even_systems(plan):
     assert shares(plan, [100, 100, 100, 100]) == (True, [38, 38, 38, 38])
     assert shares(plan, [432, 432, 106, 106], sms=100) == (True, [40, 40, 10, 10])
+
+
+@pytest.mark.parametrize("start,answers,way,tried,ok", [
+    (0, [0], 0, [0], 1), (0, [1, 0], 1, [0, 1], 1), (0, [1, 1], 2, [0, 1], 1), (1, [0], 1, [1], 1),
+    (1, [1], 2, [1], 1), (0, [2], 0, [0], 0), (0, [1, 2], 1, [0, 1], 0), (2, [], 2, [], 1)])
+def test_ways_of_a_solve(plan, start, answers, way, tried, ok):
+    """Launches that the device answers with done (0), no room (1) or another
+    error (2): a refused cluster goes to every SM, that to the graph, and an
+    error to the caller."""
+    a, t, n, w = (C.c_int * 4)(*answers), (C.c_int * 4)(), C.c_int(), C.c_int(start)
+    assert plan.ways(C.byref(w), a, t, C.byref(n)) == ok
+    assert w.value == way and list(t[:n.value]) == tried
