@@ -24,11 +24,15 @@ _L = _lib.load()
 # pointers of them) and the current stream comes as its raw handle: on short
 # vectors a BLAS-1 call is mostly this code, and stream and pointer objects
 # were a good part of it.
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+if hasattr(torch._C, "_cuda_getCurrentRawStream"):
+    _raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
+    def _stream():
+        return _raw_stream(_device())
+else:   # a torch build without CUDA: torch says so when a call asks for a stream
 
-def _stream():
-    return _raw_stream(_device())
+    def _stream():
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):

@@ -77,3 +77,21 @@ def test_build_targets_sm103a_only():
     m = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(m)
     assert m.ARCH == ["-gencode", "arch=compute_103a,code=sm_103a"]
+
+
+def test_import_without_cuda_in_torch(lib):
+    """A torch build without CUDA has no stream functions: the package still
+    imports, and a call that asks for a stream gets torch's own error."""
+    import subprocess
+    import sys
+    code = ("import torch\n"
+            "for f in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    delattr(torch._C, f)\n"
+            "import paper_2112_06465_gb300 as hz\n"
+            "torch.cuda.current_stream = lambda: 1 / 0\n"
+            "try:\n"
+            "    hz.hz._stream()\n"
+            "except ZeroDivisionError:\n"
+            "    print('asked torch')\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0 and "asked torch" in r.stdout, r.stderr
