@@ -269,3 +269,71 @@ def test_sweep_shares(hz, sizes, chip):
             assert abs(info.iters - one.iters) <= 2 + one.iters // 4
     for M in mats:
         M.close()
+
+
+# sizes whose slices do not divide among a cluster's CTAs (some own none), and
+# partial last slices; 1, 2 and 33 rows stay off the layout (padding)
+@pytest.mark.parametrize("n,chip", [
+    (1, False), (2, False), (33, False), (31, True), (32, True), (96, True), (160, True), (224, True), (290, True),
+    (479, True), (513, True), (6143, True), (6177, True)])
+def test_small_sizes_on_chip(hz, n, chip):
+    """Which of the smallest systems are solved on chip (a solve by the graph
+    gives handles of lane runs and of the unpacked kind the same sums), and
+    their solutions against the graph's."""
+    A = operator(n, n)
+    b, x0 = vec(n, n + 1), vec(n, n + 2)
+    for opt in METHODS + [dict(mode="mixed", precond="jacobi")]:
+        out = []
+        for kind in ("flat64p", "flat64"):
+            M = hz.Matrix.from_csr(A, c64=True)
+            M.set_spmv(kind)
+            out.append(hz.zsolve(M, b, x=x0.clone(), tol=TOL, maxit=200, **opt))
+            M.close()
+        (x, i), (y, j) = out
+        assert i.status == 0 and j.status == 0
+        assert float(torch.linalg.vector_norm(x - y) / torch.linalg.vector_norm(y)) <= 3.5 * TOL
+        if opt.get("mode") != "mixed":   # (complex64 products of both kinds read the slices)
+            assert torch.equal(x, y) != chip, opt
+
+
+@pytest.mark.parametrize("n", [1000, 20011])
+@pytest.mark.parametrize("opt", METHODS[:2])
+def test_history(hz, n, opt):
+    """The whole residual history against the graph's.  One step's rounding is
+    below 100 2^-53 (||A|| ||x|| + ||b||) ~ 1e-13 ||b||; the recurrences of this
+    well-conditioned operator (condition below 16) may carry it on, so the two
+    stay together within 1e-9 ||b||.  Entries past the end are not written."""
+    A, b = operator(n, 3 * n), vec(n, 3 * n + 1)
+    h = []
+    for kind in ("flat64p", "flat64"):
+        M = hz.Matrix.from_csr(A)
+        M.set_spmv(kind)
+        hist = torch.full((201,), -1.0, dtype=torch.float64, device="cuda")
+        _, info = hz.zsolve(M, b, tol=TOL, maxit=200, hist=hist, **opt)
+        assert info.status == 0 and info.restarts == 0
+        v = hist.cpu().numpy()
+        assert np.all(v[:info.iters + 1] >= 0.0) and np.all(v[info.iters + 1:] == -1.0)
+        assert v[info.iters] == info.relres_rec
+        h.append(v[:info.iters + 1])
+        M.close()
+    m = min(map(len, h))
+    assert np.all(np.abs(h[0][:m] - h[1][:m]) <= 1e-9)
+
+
+@pytest.mark.parametrize("n", [64, 9728])   # one cluster; every SM
+@pytest.mark.parametrize("opt", METHODS[:3])
+def test_breakdown(hz, n, opt):
+    """Blocks [[0, 1], [-1, 0]] with b = (1, 0) in each: <r^, A r> = 0 in the
+    first step.  The outcome is the graph's."""
+    i = np.arange(n)
+    A = W.CSR(n, np.arange(n + 1, dtype=np.int32), (i ^ 1).astype(np.int32), np.where(i % 2 == 0, 1.0, -1.0) + 0j)
+    b = torch.as_tensor(np.where(i % 2 == 0, 1.0, 0.0) + 0j).cuda()
+    out = []
+    for kind in ("flat64p", "flat64"):
+        M = hz.Matrix.from_csr(A, c64=True)
+        M.set_spmv(kind)
+        out.append(hz.zsolve(M, b, tol=TOL, maxit=50, **opt))
+        M.close()
+    (x, p), (y, q) = out
+    assert (p.status, p.iters, p.outer) == (q.status, q.iters, q.outer) and p.status in (4, 5)
+    assert p.relres_true == q.relres_true and torch.equal(x, y)
