@@ -121,7 +121,7 @@ def recorded_traffic(name):
         return None
 
 
-TRAFFIC_FILES = {4: "spmv_ffb_c2_traffic.txt", 6: "spmv_d64b_c2_traffic.txt", 7: "spmv_d64p_c2_traffic.txt"}
+TRAFFIC_FILES = {4: "spmv_ffb_c2_traffic.txt", 6: "spmv_d64b_c2_traffic.txt", 7: "spmv_sl_c2_traffic.txt"}
 
 
 class ClockSampler:
@@ -240,7 +240,8 @@ SPMV_KINDS = {0: "binary64 CSR-vector (k_spmv)", 1: "binary64 SELL-C-sigma (k_sp
               4: "double-float block-flat (k_spmv_ffb)",
               5: "double-float block-flat, bulk-copy staged (k_spmv_fft)",
               6: "binary64 block-flat, contiguous lane runs (k_spmv_d64b)",
-              7: "binary64 block-flat on the packed stream (k_spmv_d64b<packed>)"}
+              7: "binary64 on the packed copy, one row per lane (k_spmv_sl; k_spmv_d64b<packed> where row "
+                 "lengths differ too much)"}
 BINARY64_KINDS = (0, 1, 6, 7)
 # binary64 roof of GB300: the nominal FP64 rate of the profiling recipe's
 # table (1.25 TFLOP/s); an own FMA-throughput probe measured 1.05 TFLOP/s

@@ -139,8 +139,9 @@ enum {
                                 lengths the copy holds one row per lane instead, the diagonal
                                 entry last (another order of the sums within the same error
                                 bound; the few rows far longer than the others are read from
-                                the caller's arrays).  Device memory: 20 bytes per slot, about
-                                nnz slots.  The default without HZ_FLAG_FF */
+                                the caller's arrays, and so are all rows by a product of few
+                                wide slices, as HZ_SPMV_FLAT64).  Device memory: 20 bytes per
+                                slot, about nnz slots.  The default without HZ_FLAG_FF */
 };
 
 typedef struct {
@@ -320,10 +321,13 @@ typedef struct {
  *
  * d_x holds x0 on entry (unless x0_is_zero) and the solution on exit (also
  * on HZ_NOT_CONVERGED / HZ_BREAKDOWN: the last iterate).  The whole
- * iteration runs on the device inside one CUDA graph with a device-side
- * loop; the call synchronises `stream` once per (re)start and fills *h_info.
- * The handle keeps the solver workspace (7 vectors of n complex numbers,
- * plus the complex64 copies in mixed mode) and the graph between calls.
+ * iteration runs on the device: as one persistent kernel for
+ * HZ_SPMV_FLAT64P handles with one row per lane whose vectors fit into the
+ * SMs' shared memory (BiCGStab, TFQMR and mixed mode; 3 vectors of n complex
+ * numbers in device memory, 4 in mixed mode), otherwise inside one CUDA graph
+ * with a device-side loop (7 vectors, plus the complex64 copies in mixed
+ * mode).  The call synchronises `stream` once per (re)start and fills
+ * *h_info.  The handle keeps the workspace and the graph between calls.
  * Calls on the same handle must not overlap.
  * Returns the solve status (HZ_OK, HZ_NOT_CONVERGED, HZ_BREAKDOWN,
  * HZ_ERR_NAN) or an error code.
@@ -346,8 +350,9 @@ HZ_API hz_status hz_zsolve_opts(hz_mat *A, const hz_z *d_b, hz_z *d_x,
 /*
  * Solve nsys independent systems A[s] x[s] = b[s] (a frequency sweep) in one
  * persistent cooperative launch: every system keeps its own BiCGStab state
- * on the device; all systems advance together through the phases of the
- * iteration and leave the batch as they converge.  Same algorithm,
+ * on the device; they run side by side on chip where they fit (below), or
+ * advance together through the phases of the iteration and leave the batch as
+ * they converge.  Same algorithm,
  * stopping rule and status semantics as hz_zsolve (no restart), per system.
  * mode HZ_MODE_FP64: the batch runs in double-float arithmetic when every
  * handle (with n > 0) was created with HZ_FLAG_FF and its SpMV kind is a
@@ -357,8 +362,9 @@ HZ_API hz_status hz_zsolve_opts(hz_mat *A, const hz_z *d_b, hz_z *d_x,
  * at most 50 refinement steps, maxit capping the inner iterations in total,
  * the best iterate kept), each system at its own stage; the handles' complex64
  * copies are made on demand (synchronising).  Binary64 systems that fit
- * on chip together (HZ_SPMV_FLAT64P handles with one row per lane, no more
- * systems than SMs) run side by side, each on SMs of its own; the workspace
+ * on chip together (HZ_SPMV_FLAT64P handles with one row per lane; an SM for
+ * each system and enough SMs for the vectors of the large ones) run side by
+ * side, each on SMs of its own; the workspace
  * of such a sweep stays with its first handle.  Otherwise binary64 products
  * run on each handle's row blocks (the block-flat core of HZ_SPMV_FLAT64), complex64 and
  * double-float ones with `group` lanes per row.  d_x[s] holds x0 on entry and

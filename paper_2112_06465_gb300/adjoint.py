@@ -5,7 +5,7 @@ For x = A^{-1} b and the conjugate-Wirtinger gradient g = dL/dx that PyTorch
 hands to backward (for a real loss L), the adjoint system is A^H lambda = g.
 Writing mu = conj(lambda) turns it into A^T mu = conj(g); A is complex
 symmetric, so this is a second solve with the SAME operator (and the same
-captured solver graph).  Then
+solver workspace).  Then
     dL/db        = conj(mu)
     dL/dA_ij     = -conj(mu_i x_j)          (stored entries only)
     dL/dtheta_i  = conj(c) * dL/dA_ii       for A_ii = base_i + c * theta_i.

@@ -1,6 +1,9 @@
 // batched.cu -- a sweep of independent BiCGStab solves (one per frequency or
 // geometry) in ONE persistent cooperative launch.
 //
+// Binary64 systems that fit on chip together take the launch of persist.cu,
+// each on CTAs of its own; the kernels here run the other sweeps.
+//
 // Every system keeps its own BiCGStab state on the device (the Section 7
 // algorithm, as in bicgstab.cu).  All systems advance together through the
 // phases of an iteration; a phase is a list of work items (row blocks for
@@ -835,7 +838,7 @@ extern "C" HZ_API hz_status hz_zsolve_batched(int32_t nsys, hz_mat *const *A, co
         if (mixed && A[k]->n > 0) HZ_TRY(ensure_c64(A[k], s));
     }
     // binary64 systems whose vectors fit on chip: each on CTAs of its own
-    // (12 boxes of 15^3 to 24^3: 3.7 ms, in the phases below 10.4 ms); more
+    // (12 boxes of 15^3 to 24^3: 3.8 ms, in the phases below 10.4 ms); more
     // systems than SMs, larger ones and the other formats take the phases
     std::vector<int> ncta;
     if (!mixed && !ff && ps_batch_plan(A, nsys, &ncta)) {

@@ -1096,9 +1096,11 @@ static cudaError_t ps_launch(PsKind kind, hz_mat *const *A, const PsSys *h, int 
 //   BiCGStab    15.4 / 21.0  16.0 / 21.2  17.9 / 22.8  20.7 / 23.9  24.1 / 23.4  24.6* / 24.5
 //   TFQMR       15.5 / 19.3  15.1 / 20.4  17.6 / 21.5  20.8 / 22.9  24.4 / 22.8
 //   mixed        7.0 /  9.7   6.7 / 10.5   7.3 / 11.9   7.3 / 11.9   7.9 / 12.3   9.0 / 12.5
-// (* does not fit).  So up to 12 slices per CTA in binary64, 32 (as many as
-// always fit with rows of 15) in the mixed method, whose passes run on the
-// binary32 pipes.  The CTAs (0: not this way) and their shared memory:
+// (* does not fit).  So up to 12 slices per CTA in binary64, 32 in the mixed
+// method, whose passes run on the binary32 pipes, where the staged stream fits
+// beside the vectors: with 12 slices rows of up to 22 entries (TFQMR 21), with
+// 32 rows of up to 13 (28 slices with rows of 15); wider ones take every SM.
+// The CTAs (0: not this way) and their shared memory:
 static int ps_cluster(const hz_mat *A, PsKind kind, size_t *smem) {
     const PsMethod m = ps_method(kind);
     if (A->sl_long) return 0;   // (their columns are not staged)
@@ -1268,8 +1270,7 @@ hz_status ps_solve(hz_mat *A, PsKind kind, const Ctl &c, Info *out, int *restart
 // The systems run at their own pace, each with barriers among its own CTAs
 // only, instead of advancing together through grid-wide phases
 // (batched.cu, 75 to 95 us per iteration for any sweep of small systems).
-// CTAs are shared out by rows, one more at a time to the system whose CTAs
-// own the most slices.  Twelve boxes of 15^3 to 24^3 unknowns: 10.4 -> 3.7 ms.
+// CTAs are shared out by rows (sweep_plan).  Twelve boxes of 15^3 to 24^3 unknowns: 10.4 -> 3.8 ms.
 struct PsBatch {
     std::atomic_flag busy = ATOMIC_FLAG_INIT;
     void *mem = nullptr;
